@@ -159,8 +159,9 @@ bool is_repspc(const std::vector<HostOp> &ops, size_t i) {
 }
 
 // The register-subtree operation i (inside a subtree entered at o0 with n0
-// leaves) as a RegSub call; returns the number of list entries it covers
-// (5 for a fused Repetition-SPC node).
+// leaves) as a RegSub call; returns the number of list entries it covers: 5 for
+// a fused Repetition-SPC node, 2 for a G whose right child is a Rate-1 node (the
+// child's LLRs are used for their signs only).
 size_t emit_reg_op(std::ostream &o, const std::vector<HostOp> &ops, size_t i, uint32_t o0,
                    const char *indent) {
     const HostOp &op = ops[i];
@@ -170,66 +171,24 @@ size_t emit_reg_op(std::ostream &o, const std::vector<HostOp> &ops, size_t i, ui
         return 5;
     }
     o << indent << "r.template ";
+    if (op.kind == OP_G && ops[i + 1].kind == OP_R1 && ops[i + 1].log2n + 1 == op.log2n) {
+        o << "g_r1<" << n << "u, " << p << "u>();\n";
+        return 2;
+    }
     switch (op.kind) {
     case OP_F:
     case OP_G:
     case OP_G0R: o << "fg<" << kind_name(op.kind) << ", " << n << "u, " << p << "u>();\n"; break;
     case OP_C: o << "combine<" << n << "u, " << p << "u, false>();\n"; break;
     case OP_C0R: o << "combine<" << n << "u, " << p << "u, true>();\n"; break;
-    case OP_R0: o << "r0<" << n << "u, " << p << "u>();\n"; break;
+    case OP_R0:  // inside a subtree always a right child
+        o << ((op.flags & OPW_REG_ENTER) ? "r0<" : "r0_right<") << n << "u, " << p << "u>();\n";
+        break;
     case OP_R1: o << "r1<" << n << "u, " << p << "u>();\n"; break;
     case OP_REP: o << "rep<" << n << "u, " << p << "u>();\n"; break;
     default: o << "spc<" << n << "u, " << p << "u>();\n"; break;
     }
     return 1;
-}
-
-// In the per-lane form (kLocalLeaves), a split node of 4 to 16 leaves inside a
-// register subtree is decoded by every lane on its own (RegSub::lenter, lfg,
-// lr1, lrep, lspc; Combine and Rate-0 are the same word operations). If
-// operation i starts such a node, emits the node's operations in that form and
-// returns how many list entries it covered; otherwise 0.
-size_t emit_local_node(std::ostream &o, const std::vector<HostOp> &ops, size_t i, uint32_t o0,
-                       const char *indent) {
-    const HostOp &a = ops[i];
-    const uint32_t n = 1u << a.log2n;
-    if ((a.kind != OP_F && a.kind != OP_G0R) || n > 16 || n < 4 || (a.flags & OPW_REG_ENTER))
-        return 0;
-    size_t j = i + 1;  // the node's operations: offsets inside [off, off + n), sizes <= n
-    while (j < ops.size() && (ops[j].flags & OPW_REG) && !(ops[j].flags & OPW_REG_ENTER) &&
-           ops[j].off >= a.off && ops[j].off < a.off + n && ops[j].log2n <= a.log2n)
-        ++j;
-    for (size_t k = i; k < j; ++k)
-        if (ops[k].flags & OPW_REG_EXIT) return 0;  // the node is the subtree itself
-    o << indent << "r.template lenter<" << n << "u>();\n";
-    for (size_t k = i; k < j; ++k) {
-        const HostOp &op = ops[k];
-        const uint32_t m = 1u << op.log2n, p = op.off - o0;
-        o << indent << "r.template ";
-        switch (op.kind) {
-        case OP_F:
-        case OP_G:
-        case OP_G0R: o << "lfg<" << kind_name(op.kind) << ", " << m << "u, " << p << "u>();\n"; break;
-        case OP_C: o << "combine<" << m << "u, " << p << "u, false>();\n"; break;
-        case OP_C0R: o << "combine<" << m << "u, " << p << "u, true>();\n"; break;
-        case OP_R0: o << "r0<" << m << "u, " << p << "u>();\n"; break;
-        case OP_R1: o << "lr1<" << m << "u, " << p << "u>();\n"; break;
-        case OP_REP: o << "lrep<" << m << "u, " << p << "u>();\n"; break;
-        default: o << "lspc<" << m << "u, " << p << "u>();\n"; break;
-        }
-    }
-    return j - i;
-}
-
-// One register-subtree operation (or a per-lane node, or a fused
-// Repetition-SPC node) at list index i; returns the entries covered.
-size_t emit_reg_ops(std::ostream &o, const std::vector<HostOp> &ops, size_t i, uint32_t o0,
-                    const char *indent, bool local) {
-    if (local) {
-        const size_t used = emit_local_node(o, ops, i, o0, indent);
-        if (used) return used;
-    }
-    return emit_reg_op(o, ops, i, o0, indent);
 }
 
 // Compact form: one out-of-line function per distinct register subtree (the
@@ -240,7 +199,7 @@ size_t emit_reg_ops(std::ostream &o, const std::vector<HostOp> &ops, size_t i, u
 // subtrees of different codes share one function; nullptr for a map of its own.
 std::map<size_t, size_t> emit_subtree_functions(std::ostringstream &o, const std::vector<HostOp> &ops,
                                                 const char *T, uint32_t R,
-                                                const std::string &prefix, bool local,
+                                                const std::string &prefix,
                                                 std::map<std::string, size_t> *shared = nullptr) {
     std::map<std::string, size_t> own;
     std::map<std::string, size_t> &ids = shared ? *shared : own;
@@ -250,7 +209,7 @@ std::map<size_t, size_t> emit_subtree_functions(std::ostringstream &o, const std
         const uint32_t o0 = ops[i].off, n0 = 1u << ops[i].log2n;
         std::ostringstream b;
         for (size_t j = i;;) {
-            const size_t used = emit_reg_ops(b, ops, j, o0, "  ", local);
+            const size_t used = emit_reg_op(b, ops, j, o0, "  ");
             j += used;
             if (ops[j - 1].flags & OPW_REG_EXIT) break;
         }
@@ -261,7 +220,7 @@ std::map<size_t, size_t> emit_subtree_functions(std::ostringstream &o, const std
             it = ids.emplace(key, id).first;
             o << "__device__ __noinline__ void " << prefix << "sub" << id << "(const " << T
               << " *in, uint32_t *beta, uint32_t o0) {\n"
-              << "  RegSub<" << T << ", " << R << "u> r;\n  r.lane = threadIdx.x & 31u;\n"
+              << "  RegSub<" << T << ", " << R << "u, 32u> r;\n"
               << "  r.template enter<" << n0 << "u>(in);\n" << b.str()
               << "  r.template exit<" << n0 << "u>(beta, o0);\n}\n";
         }
@@ -324,7 +283,6 @@ void emit_body(std::ostringstream &o, const polar_code &code, bool is_i8, uint32
                bool warp_frames = false, bool chan_global = true,
                std::map<std::string, size_t> *shared_subs = nullptr) {
     const bool outline_sub = outline & kOutlineSubtrees, outline_mem = outline & kOutlineMemory;
-    const bool local = outline & kLocalLeaves;
     const uint32_t N = code.N;
     const std::vector<HostOp> ops = code.build_ops(R);
     const std::vector<std::vector<uint32_t>> prefetch = plan_prefetch(ops, N, S, chan_global);
@@ -365,7 +323,7 @@ void emit_body(std::ostringstream &o, const polar_code &code, bool is_i8, uint32
     const char *T = is_i8 ? "int8_t" : "float";
     std::map<size_t, size_t> sub_at;
     const std::string sub_prefix = shared_subs ? std::string("Shared_") : name + "_";
-    if (outline_sub) sub_at = emit_subtree_functions(o, ops, T, R, sub_prefix, local, shared_subs);
+    if (outline_sub) sub_at = emit_subtree_functions(o, ops, T, R, sub_prefix, shared_subs);
     o << "struct " << name << " {\n"
       << "  __device__ __forceinline__ void operator()(const Frame<" << T << "> &fr, float *) const {\n"
       << "    using T = " << T << ";\n"
@@ -536,10 +494,10 @@ void emit_body(std::ostringstream &o, const polar_code &code, bool is_i8, uint32
         if (op.flags & OPW_REG_ENTER) {
             o0 = op.off;
             n0 = n;
-            o << "      {\n        RegSub<T, " << R << "u> r;\n        r.lane = lane;\n"
+            o << "      {\n        RegSub<T, " << R << "u, 32u> r;\n"
               << "        r.template enter<" << n0 << "u>(" << in(n0) << ");\n";
         }
-        i += emit_reg_ops(o, ops, i, o0, "        ", local) - 1;
+        i += emit_reg_op(o, ops, i, o0, "        ") - 1;
         if (ops[i].flags & OPW_REG_EXIT) {
             o << "        r.template exit<" << n0 << "u>(fr.beta, " << o0 << "u);\n      }\n"
               << "      __syncwarp();\n" << align;

@@ -689,7 +689,6 @@ polar_status polar_code_compile_ex(polar_code_t *code, int is_i8, size_t n_frame
     const uint32_t form = flags & (POLAR_COMPILE_COMPACT | POLAR_COMPILE_FULL);
     uint32_t outline = flags & POLAR_COMPILE_COMPACT;  // subtrees (1) and/or memory ops (2)
     if (!form && code->ops.size() > kCompactOps) outline = kOutlineSubtrees | kOutlineMemory;
-    if (flags & POLAR_COMPILE_LOCAL_LEAVES) outline |= kLocalLeaves;
     if (reg_subtree == 0) reg_subtree = 256;
     if (!is_pow2(reg_subtree) || reg_subtree < 32 || reg_subtree > 1024) return POLAR_EINVAL;
     int device = -1;

@@ -1243,133 +1243,252 @@ __device__ __forceinline__ void static_for(F &&f) {
     }
 }
 
-// Register-subtree arithmetic. Both LLR types are held in float registers:
-// int8 LLRs are integers in [-127, 127], exact in float, and every sum of two
-// of them is exact too. int8 keeps its saturation: each G and each Repetition
-// fold is clamped to [-127, 127], which is what the saturating byte add
-// followed by max(-127) gives. F is one min.xorsign.abs for both types.
-template <typename T>
-__device__ __forceinline__ float sat_reg(float v) {
-    if constexpr (sizeof(T) == 1) return fminf(fmaxf(v, -127.0f), 127.0f);
-    else return v;
-}
-template <typename T>
-__device__ __forceinline__ float rop_f(float a, float b) { return f_f32(a, b); }
-template <typename T>
-__device__ __forceinline__ float rop_g(float a, float b, uint32_t bit) { return sat_reg<T>(g_f32(a, b, bit)); }
-template <typename T>
-__device__ __forceinline__ float rop_add(float a, float b) { return sat_reg<T>(a + b); }
+// Register-subtree values. A 32-bit register holds W values of one lane: one
+// float (W = 1), or for int8 LLRs two f16 (W = 2; integers of magnitude <= 254
+// are exact in f16, see op_i8x4). int8 keeps its saturation: every sum is
+// clamped to [-127, 127], which is what the saturating byte add followed by
+// max(-127) gives. Bits are sign bits (SGN): beta = 1 is a set sign, so G flips
+// signs with one XOR and a hard decision is the sign of x + 0, which is set
+// exactly when x < 0 (-0 + 0 = +0, and a NaN sum is the positive NaN).
+template <typename T> struct SubVal;
+template <> struct SubVal<float> {
+    static constexpr uint32_t W = 1, SGN = 0x80000000u;
+    __device__ static __forceinline__ uint32_t f(uint32_t a, uint32_t b) {
+        return __float_as_uint(f_f32(__uint_as_float(a), __uint_as_float(b)));
+    }
+    __device__ static __forceinline__ uint32_t add(uint32_t a, uint32_t b) {
+        return __float_as_uint(__uint_as_float(a) + __uint_as_float(b));
+    }
+    __device__ static __forceinline__ uint32_t add_sign(uint32_t a, uint32_t b) { return hard(add(a, b)); }
+    __device__ static __forceinline__ uint32_t hard(uint32_t a) {
+        return __float_as_uint(__uint_as_float(a) + 0.0f);
+    }
+};
+template <> struct SubVal<int8_t> {
+    static constexpr uint32_t W = 2, SGN = 0x80008000u;
+    __device__ static __forceinline__ uint32_t f(uint32_t a, uint32_t b) { return hf2(a, b); }
+    __device__ static __forceinline__ uint32_t add(uint32_t a, uint32_t b) { return hsat2(hadd2(a, b)); }
+    // a sum of which only the hard decision is used: the clamp keeps the sign
+    __device__ static __forceinline__ uint32_t add_sign(uint32_t a, uint32_t b) { return hard(hadd2(a, b)); }
+    __device__ static __forceinline__ uint32_t hard(uint32_t a) { return hadd2(a, 0u); }
+};
 
-// Subtree of at most R leaves decoded by warp 0 with compile-time node sizes and
-// offsets (the generated decoders): stage m >= 32 is m/32 registers per lane
-// (element j + 32k in register k of lane j), stages 1..16 share register A
-// (stage m element j on lane m + j), and the subtree's bits are R/32 words held
-// identically by every lane (word k = leaves [32k, 32k + 32) of the subtree).
-// F and G above 32 leaves are lane-local; at 32 and below they are shuffles.
-template <typename T, uint32_t R>
+// Unsigned type of G bits (the bits of one chunk of a frame's values).
+template <uint32_t G> struct BetaUnit { using type = uint8_t; };
+template <> struct BetaUnit<16> { using type = unsigned short; };
+
+__host__ __device__ constexpr uint32_t clog2(uint32_t v) { return v <= 1 ? 0u : 1u + clog2(v / 2); }
+
+// Subtree of at most R leaves decoded in registers with compile-time node sizes
+// and offsets (the generated decoders), G lanes per frame: G = 32 is one frame
+// per warp; with G = 8 or 16 one warp decodes the same subtree of 32 / G frames
+// at once, lanes [gG, gG + G) holding frame g.
+//
+// Layout. A row is one register per lane: E = G W values of a node. Value e of
+// a stage of n >= E values sits in row e / E, half (e / G) % W, lane e % G, so F
+// and G of nodes of 2E and more values are lane-local. At n = E with W = 2 the
+// two operands are the halves of one register. A stage of n <= G values is
+// kept replicated: every lane li (and both halves) holds value li % n. Then the
+// partner operand of F and G is one shuffle away (lane li ^ n/2), is kept from F
+// for the G of the same node, no lane idles and none needs a predicate, every
+// lane ends a Repetition fold with the sum, Combine is one logic instruction
+// and a Rate-1 node one addition. (Before: stage n on lanes n..2n-1 and bits in
+// a word common to the warp, with two shuffles and a select for F and for G, and
+// a ballot and a bit-field insert for every node.) The narrow nodes (n <= 32)
+// are nine tenths of a frame's operations and set both the length of a frame's
+// serial chain and, through their instructions, the rate of a full GPU.
+// Measured before and after this layout (int8 unless named): one frame of
+// (32768, 29492) 77.9 -> 67.8 us, 4096 of them 352 -> 327 us (float32 883 -> 829),
+// 2,001 frames of (2048, 1707) 24.6 -> 20.5 us.
+template <typename T, uint32_t R, uint32_t G>
 struct RegSub {
-    using Acc = float;  // both LLR types (see rop_f)
-    static constexpr uint32_t NWORD = R >= 32 ? R / 32 : 1;
-    Acc s1024[32], s512[16], s256[8], s128[4], s64[2], s32, A;
-    Acc l16[16], l8[8], l4[4], l2[2], l1;  // the per-lane form of nodes of <= 16 leaves
-    uint32_t bw[NWORD];
-    uint32_t lane;
+    using V = SubVal<T>;
+    static constexpr uint32_t W = V::W, SGN = V::SGN, E = G * W;
+    static constexpr uint32_t NR = R >= E ? R / E : 1;
+    uint32_t v32[32], v16[16], v8[8], v4[4], v2[2], v1;  // stages of n >= E values: n / E rows
+    uint32_t t[7], y[7];       // stage 2^k < E (replicated); partner operand of node 2^k <= E
+    uint32_t B[NR];            // bits of nodes of n >= E values, by row
+    uint32_t bl[7], br[7];     // bits of left / right nodes of 2^k < E values (replicated)
+    uint32_t ca[5], cb[5];     // sign mask on lanes with bit k of the lane index clear / set
+    uint32_t li, gsh;          // lane within the frame, first lane of the frame
 
-    template <uint32_t m, uint32_t k>
-    __device__ __forceinline__ Acc &reg() {
-        if constexpr (m == 1024) return s1024[k];
-        else if constexpr (m == 512) return s512[k];
-        else if constexpr (m == 256) return s256[k];
-        else if constexpr (m == 128) return s128[k];
-        else if constexpr (m == 64) return s64[k];
-        else return s32;
+    __device__ __forceinline__ void init() {
+        const uint32_t lane = threadIdx.x & 31u;
+        li = lane & (G - 1u);
+        gsh = lane & ~(G - 1u);
+        static_for<0, 5>([&](auto kc) {
+            constexpr uint32_t k = decltype(kc)::value;
+            ca[k] = (lane >> k) & 1u ? 0u : SGN;
+            cb[k] = SGN ^ ca[k];
+        });
     }
 
-    // Load the subtree root's LLRs (stage n0) from memory.
+    template <uint32_t n, uint32_t k>
+    __device__ __forceinline__ uint32_t &row() {
+        if constexpr (n < E) return t[clog2(n)];
+        else if constexpr (n / E == 32) return v32[k];
+        else if constexpr (n / E == 16) return v16[k];
+        else if constexpr (n / E == 8) return v8[k];
+        else if constexpr (n / E == 4) return v4[k];
+        else if constexpr (n / E == 2) return v2[k];
+        else return v1;
+    }
+    // Bits of node (n, p), n < E (or its row when n = E).
+    template <uint32_t n, uint32_t p>
+    __device__ __forceinline__ uint32_t &bits() {
+        if constexpr (n >= E) return B[p / E];
+        else if constexpr ((p & n) != 0) return br[clog2(n)];
+        else return bl[clog2(n)];
+    }
+    // The other operand's lanes for a node of n <= E values.
+    template <uint32_t n>
+    __device__ __forceinline__ uint32_t partner(uint32_t x) {
+        if constexpr (W == 2 && n == E) return prmt(x, x, 0x1032u);
+        else return __shfl_xor_sync(kFull, x, n / 2);
+    }
+    // Sign mask of the values that are operand a (index < n/2) / b of a node of n <= E.
+    template <uint32_t n>
+    __device__ __forceinline__ uint32_t mask_a() {
+        if constexpr (W == 2 && n == E) return 0x00008000u;
+        else return ca[clog2(n) - 1];
+    }
+    template <uint32_t n>
+    __device__ __forceinline__ uint32_t mask_b() {
+        if constexpr (W == 2 && n == E) return 0x80000000u;
+        else return cb[clog2(n) - 1];
+    }
+    // Bit (lowest value first) mask of a replicated node's n <= G lanes of this frame.
+    template <uint32_t n>
+    __device__ __forceinline__ uint32_t of_frame(uint32_t ballot) {
+        if constexpr (G == 32) return n == 32 ? ballot : (ballot & ((1u << n) - 1u));
+        else return (ballot >> gsh) & ((1u << n) - 1u);
+    }
+    __device__ __forceinline__ uint32_t min_over_frame(uint32_t x, uint32_t n) {
+        if constexpr (G == 32) return __reduce_min_sync(kFull, x);
+#pragma unroll
+        for (uint32_t m = G / 2; m >= 1; m /= 2)
+            if (m < n) x = min(x, __shfl_xor_sync(kFull, x, m));
+        return x;
+    }
+
+    // Load the subtree root's LLRs (stage n0) of this lane's frame.
     template <uint32_t n0>
     __device__ __forceinline__ void enter(const T *src) {
-        if constexpr (n0 >= 32) {
-            static_for<0, n0 / 32>([&](auto kc) {
+        init();
+        if constexpr (n0 >= E) {
+            static_for<0, n0 / E>([&](auto kc) {
                 constexpr uint32_t k = decltype(kc)::value;
-                reg<n0, k>() = static_cast<Acc>(src[32 * k + lane]);
+                if constexpr (W == 1) row<n0, k>() = __float_as_uint(src[E * k + li]);
+                else row<n0, k>() = pair(src[E * k + li], src[E * k + G + li]);
             });
         } else {
-            A = (lane >= n0 && lane < 2 * n0) ? static_cast<Acc>(src[(lane - n0) & 31u]) : Acc(0);
+            const T x = src[li & (n0 - 1u)];
+            if constexpr (W == 1) t[clog2(n0)] = __float_as_uint(x);
+            else t[clog2(n0)] = pair(x, x);
         }
     }
+    // Two int8 values as f16x2: 0x6480 + x is the f16 1152 + x (x in [-127, 127]
+    // keeps the exponent), and the sum of the two halves never carries.
+    __device__ static __forceinline__ uint32_t pair(int32_t lo, int32_t hi) {
+        return hadd2(0x64806480u + static_cast<uint32_t>(lo) + (static_cast<uint32_t>(hi) << 16),
+                     0xE480E480u);
+    }
 
-    // Store the subtree's n0 bits at leaf offset o0 of beta. The words are the
-    // same on every lane, so lane 0 stores them, 16 bytes at a time (o0 is a
-    // multiple of n0, so the words are 16-byte aligned from 128 leaves up).
+    // Store the subtree's n0 bits at leaf offset o0 of this lane's frame's beta.
     template <uint32_t n0>
     __device__ __forceinline__ void exit(uint32_t *beta, uint32_t o0) {
-        if constexpr (n0 >= 128) {
-            if (lane == 0) {
-                static_for<0, n0 / 128>([&](auto kc) {
-                    constexpr uint32_t k = decltype(kc)::value;
-                    uint4 q;
-                    q.x = bw[4 * k];
-                    q.y = bw[4 * k + 1];
-                    q.z = bw[4 * k + 2];
-                    q.w = bw[4 * k + 3];
-                    *reinterpret_cast<uint4 *>(beta + (o0 >> 5) + 4 * k) = q;
-                });
+        if constexpr (n0 < E) {
+            const uint32_t m = of_frame<n0>(__ballot_sync(kFull, (bl[clog2(n0)] & 0x80000000u) != 0u));
+            if (li == 0) {
+                if constexpr (G == 32) {
+                    write_field(beta, o0, n0, m);
+                } else if constexpr (n0 < 8) {
+                    write_field(beta, o0, n0, m);
+                } else {
+                    uint8_t *b = reinterpret_cast<uint8_t *>(beta) + (o0 >> 3);
+                    b[0] = static_cast<uint8_t>(m);
+                    if constexpr (n0 == 16) b[1] = static_cast<uint8_t>(m >> 8);
+                }
             }
-        } else if constexpr (n0 >= 32) {
-            if (lane == 0) {
+        } else if constexpr (G == 32) {
+            uint32_t w[n0 / 32];
+            static_for<0, n0 / 32>([&](auto kc) {
+                constexpr uint32_t k = decltype(kc)::value;
+                constexpr uint32_t m = (W == 2 && k % 2 == 0) ? 0x8000u : 0x80000000u;
+                w[k] = __ballot_sync(kFull, (B[k / W] & m) != 0u);
+            });
+            if (li == 0) {  // the words are the same on every lane: 16-byte stores
                 static_for<0, n0 / 32>([&](auto kc) {
                     constexpr uint32_t k = decltype(kc)::value;
-                    beta[(o0 >> 5) + k] = bw[k];
+                    if constexpr (n0 >= 128) {
+                        if constexpr (k % 4 == 0)
+                            *reinterpret_cast<uint4 *>(beta + (o0 >> 5) + k) =
+                                make_uint4(w[k], w[k + 1], w[k + 2], w[k + 3]);
+                    } else {
+                        beta[(o0 >> 5) + k] = w[k];
+                    }
                 });
             }
         } else {
-            if (lane == 0) write_field(beta, o0, n0, bw[0]);
+            // chunk k (values [kG, kG + G)) of every frame is one ballot; lane li of
+            // a frame stores chunks li, li + G, ... as G-bit units
+            using U = typename BetaUnit<G>::type;
+            U *b = reinterpret_cast<U *>(beta) + o0 / G;
+            constexpr uint32_t NC = n0 / G, STEP = NC < G ? NC : G;
+            static_for<0, NC / STEP>([&](auto qc) {
+                constexpr uint32_t q = decltype(qc)::value;
+                uint32_t mine = 0;
+                static_for<0, STEP>([&](auto kc) {
+                    constexpr uint32_t k = q * STEP + decltype(kc)::value;
+                    constexpr uint32_t m = (W == 2 && k % 2 == 0) ? 0x8000u : 0x80000000u;
+                    const uint32_t w = __ballot_sync(kFull, (B[k / W] & m) != 0u);
+                    if (li == decltype(kc)::value) mine = w;
+                });
+                if (li < STEP) b[q * STEP + li] = static_cast<U>(mine >> gsh);
+            });
         }
     }
-
-    template <uint32_t w, uint32_t q, uint32_t width>
-    __device__ __forceinline__ void set_field(uint32_t v) {
-        if constexpr (width >= 32) {
-            bw[w] = v;
-        } else {
-            constexpr uint32_t fm = ((1u << width) - 1u) << q;
-            bw[w] = (bw[w] & ~fm) | ((v << q) & fm);
-        }
-    }
-
     // F / G / G_0R of a node of n leaves at subtree offset p.
     template <uint32_t KIND, uint32_t n, uint32_t p>
     __device__ __forceinline__ void fg() {
-        if constexpr (n >= 64) {
-            constexpr uint32_t K = n / 64;
+        if constexpr (n >= 2 * E) {
+            constexpr uint32_t K = n / (2 * E);
             static_for<0, K>([&](auto kc) {
                 constexpr uint32_t k = decltype(kc)::value;
-                const Acc x = reg<n, k>(), y = reg<n, k + K>();
-                Acc r;
-                if constexpr (KIND == OP_F) r = rop_f<T>(x, y);
-                else if constexpr (KIND == OP_G) r = rop_g<T>(x, y, (bw[p / 32 + k] >> lane) & 1u);
-                else r = rop_add<T>(x, y);
-                reg<n / 2, k>() = r;
+                const uint32_t a = row<n, k>(), b = row<n, k + K>();
+                uint32_t r;
+                if constexpr (KIND == OP_F) r = V::f(a, b);
+                else if constexpr (KIND == OP_G) r = V::add(b, a ^ (B[p / E + k] & SGN));
+                else r = V::add(b, a);
+                row<n / 2, k>() = r;
             });
-        } else if constexpr (n == 32) {
-            // output element i = lane - 16 (lanes 16..31) from s32 of lanes i and i + 16
-            const Acc x = __shfl_up_sync(kFull, s32, 16);
-            const Acc y = s32;
-            Acc r;
-            if constexpr (KIND == OP_F) r = rop_f<T>(x, y);
-            else if constexpr (KIND == OP_G) r = rop_g<T>(x, y, (bw[p / 32] >> ((lane - 16) & 31u)) & 1u);
-            else r = rop_add<T>(x, y);
-            if (lane >= 16) A = r;
         } else {
-            constexpr uint32_t h = n / 2, q = p % 32;
-            // output element i = lane - h (lanes [h, 2h)) from lanes n + i and n + i + h
-            const Acc x = __shfl_down_sync(kFull, A, h);
-            const Acc y = __shfl_down_sync(kFull, A, n);
-            Acc r;
-            if constexpr (KIND == OP_F) r = rop_f<T>(x, y);
-            else if constexpr (KIND == OP_G) r = rop_g<T>(x, y, (bw[p / 32] >> ((q + lane - h) & 31u)) & 1u);
-            else r = rop_add<T>(x, y);
-            if (lane >= h && lane < 2 * h) A = r;
+            const uint32_t x = row<n, 0>();
+            if constexpr (KIND == OP_G) {
+                const uint32_t w = bits<n / 2, p>(), z = y[clog2(n)];
+                row<n / 2, 0>() = V::add(x ^ (w & mask_a<n>()), z ^ (w & mask_b<n>()));
+            } else {
+                const uint32_t z = partner<n>(x);
+                y[clog2(n)] = z;
+                row<n / 2, 0>() = KIND == OP_F ? V::f(x, z) : V::add(x, z);
+            }
+        }
+    }
+
+    // G of a node of n leaves at p and the Rate-1 decision of its right child in one.
+    template <uint32_t n, uint32_t p>
+    __device__ __forceinline__ void g_r1() {
+        constexpr uint32_t h = n / 2;
+        if constexpr (n >= 2 * E) {
+            constexpr uint32_t K = n / (2 * E);
+            static_for<0, K>([&](auto kc) {
+                constexpr uint32_t k = decltype(kc)::value;
+                B[(p + h) / E + k] = V::add_sign(row<n, k + K>(), row<n, k>() ^ (B[p / E + k] & SGN));
+            });
+        } else {
+            const uint32_t w = bits<h, p>();
+            bits<h, p + h>() = V::add_sign(row<n, 0>() ^ (w & mask_a<n>()),
+                                           y[clog2(n)] ^ (w & mask_b<n>()));
         }
     }
 
@@ -1377,227 +1496,171 @@ struct RegSub {
     template <uint32_t n, uint32_t p, bool copy>
     __device__ __forceinline__ void combine() {
         constexpr uint32_t h = n / 2;
-        if constexpr (h >= 32) {
-            static_for<0, h / 32>([&](auto kc) {
+        if constexpr (n >= 2 * E) {
+            static_for<0, h / E>([&](auto kc) {
                 constexpr uint32_t k = decltype(kc)::value;
-                const uint32_t r = bw[(p + h) / 32 + k];
-                bw[p / 32 + k] = copy ? r : (bw[p / 32 + k] ^ r);
+                const uint32_t r = B[(p + h) / E + k];
+                B[p / E + k] = copy ? r : (B[p / E + k] ^ r);
             });
         } else {
-            constexpr uint32_t w = p / 32, q = p % 32, m = (1u << h) - 1u;
-            const uint32_t l = (bw[w] >> q) & m, r = (bw[w] >> (q + h)) & m;
-            set_field<w, q, h>(copy ? r : (l ^ r));
+            const uint32_t r = bits<h, p + h>();
+            bits<n, p>() = copy ? r : (r ^ (bits<h, p>() & mask_a<n>()));
         }
     }
 
+    // Rate-0 subtree root of n leaves.
     template <uint32_t n, uint32_t p>
     __device__ __forceinline__ void r0() {
-        if constexpr (n >= 32) {
-            static_for<0, n / 32>([&](auto kc) { bw[p / 32 + decltype(kc)::value] = 0u; });
+        if constexpr (n >= E) {
+            static_for<0, n / E>([&](auto kc) { B[p / E + decltype(kc)::value] = 0u; });
         } else {
-            set_field<p / 32, p % 32, n>(0u);
+            bits<n, p>() = 0u;
         }
+    }
+    // Rate-0 right child (n leaves at p) of a split node, which has no Combine:
+    // the parent's left bits stay, its right bits are zero.
+    template <uint32_t n, uint32_t p>
+    __device__ __forceinline__ void r0_right() {
+        if constexpr (n >= E) r0<n, p>();
+        else bits<2 * n, p - n>() = bits<n, p - n>() & mask_a<2 * n>();
     }
 
     template <uint32_t n, uint32_t p>
     __device__ __forceinline__ void r1() {
-        if constexpr (n >= 32) {
-            static_for<0, n / 32>([&](auto kc) {
+        if constexpr (n >= E) {
+            static_for<0, n / E>([&](auto kc) {
                 constexpr uint32_t k = decltype(kc)::value;
-                bw[p / 32 + k] = __ballot_sync(kFull, reg<n, k>() < Acc(0));
+                B[p / E + k] = V::hard(row<n, k>());
             });
         } else {
-            const bool in = lane >= n && lane < 2 * n;
-            set_field<p / 32, p % 32, n>(__ballot_sync(kFull, in && A < Acc(0)) >> n);
+            bits<n, p>() = V::hard(t[clog2(n)]);
         }
     }
 
-    // Folds t[k] <- t[k] + t[k + m] for m = K/2, ..., 1 over K lane-local values.
+    // Folds a[k] <- a[k] + a[k + m] for m = K/2, ..., 1 over K rows.
     template <uint32_t K>
-    __device__ __forceinline__ void fold_local(Acc (&t)[K]) {
+    __device__ __forceinline__ void fold_rows(uint32_t (&a)[K]) {
         if constexpr (K > 1) {
             static_for<0, K / 2>([&](auto kc) {
                 constexpr uint32_t k = decltype(kc)::value;
-                t[k] = rop_add<T>(t[k], t[k + K / 2]);
+                a[k] = V::add(a[k], a[k + K / 2]);
             });
-            fold_local<K / 2>(reinterpret_cast<Acc(&)[K / 2]>(t));
+            fold_rows<K / 2>(reinterpret_cast<uint32_t(&)[K / 2]>(a));
         }
     }
-
+    // Repetition sum of a node of n <= E values x: t[i] + t[i + m] for m = n/2 .. 1,
+    // on every lane (a + b = b + a, so partners agree); the sign of its sum + 0.
+    template <uint32_t n>
+    __device__ __forceinline__ uint32_t rep_small(uint32_t x) {
+        static_for<0, clog2(n)>([&](auto kc) {
+            constexpr uint32_t m = n >> decltype(kc)::value;
+            x = V::add(x, partner<m>(x));
+        });
+        return V::hard(x);
+    }
     template <uint32_t n, uint32_t p>
     __device__ __forceinline__ void rep() {
-        Acc x;
-        if constexpr (n >= 32) {
-            constexpr uint32_t K = n / 32;
-            Acc t[K];
+        if constexpr (n >= E) {
+            constexpr uint32_t K = n / E;
+            uint32_t a[K];
             static_for<0, K>([&](auto kc) {
                 constexpr uint32_t k = decltype(kc)::value;
-                t[k] = reg<n, k>();
+                a[k] = row<n, k>();
             });
-            // lane-local folds t[e] += t[e + m] for m = n/2 .. 32 (e = lane + 32k)
-            fold_local<K>(t);
-            x = t[0];
-#pragma unroll
-            for (uint32_t m = 16; m >= 1; m /= 2) {
-                const Acc y = __shfl_down_sync(kFull, x, m);
-                if (lane < m) x = rop_add<T>(x, y);
-            }
-            x = __shfl_sync(kFull, x, 0);
-            const uint32_t word = x < Acc(0) ? kFull : 0u;
-            static_for<0, n / 32>([&](auto kc) { bw[p / 32 + decltype(kc)::value] = word; });
+            fold_rows<K>(a);
+            const uint32_t w = rep_small<E>(a[0]);
+            static_for<0, K>([&](auto kc) { B[p / E + decltype(kc)::value] = w; });
         } else {
-            x = A;
-#pragma unroll
-            for (uint32_t m = n / 2; m >= 1; m /= 2) {
-                const Acc y = __shfl_down_sync(kFull, x, m);
-                if (lane >= n && lane < n + m) x = rop_add<T>(x, y);
-            }
-            x = __shfl_sync(kFull, x, n);
-            set_field<p / 32, p % 32, n>(x < Acc(0) ? kFull : 0u);
+            bits<n, p>() = rep_small<n>(t[clog2(n)]);
         }
     }
 
-    // ---- Per-lane form of a node of at most 16 leaves: every lane copies the
-    // node's LLRs and decodes the whole node on its own, with no shuffles. Each
-    // operation is the same arithmetic in the same order as its shuffle form
-    // (F, G, the Repetition fold t[i] + t[i + m], the lowest-index SPC flip),
-    // and the bits land in the same warp-uniform words. Fewer dependent steps
-    // per operation than the shuffle form, more instructions: for one frame
-    // in flight (latency), not for many.
-    template <uint32_t m, uint32_t k>
-    __device__ __forceinline__ Acc &loc() {
-        if constexpr (m == 16) return l16[k];
-        else if constexpr (m == 8) return l8[k];
-        else if constexpr (m == 4) return l4[k];
-        else if constexpr (m == 2) return l2[k];
-        else return l1;
+    // SPC bits of a replicated node of n <= G values x. float32: the least
+    // magnitude over the frame's lanes, then its lowest lane (Listing 2); int8:
+    // magnitude and index fit one key. The flip is a left shift that brings the
+    // chosen value's mask bit to the sign.
+    template <uint32_t n>
+    __device__ __forceinline__ uint32_t spc_small(uint32_t x) {
+        const uint32_t d = V::hard(x), e = li & (n - 1u);
+        const uint32_t odd = __popc(of_frame<n>(__ballot_sync(kFull, static_cast<int32_t>(d) < 0))) & 1u;
+        if constexpr (W == 1) {
+            const uint32_t mag = x & 0x7fffffffu, mn = min_over_frame(mag, n);
+            const uint32_t at = of_frame<n>(__ballot_sync(kFull, mag == mn));
+            const uint32_t pick = at & (0u - at) & (0u - odd);
+            return d ^ ((pick << (31u - e)) & SGN);
+        } else {
+            const uint32_t key = (x & 0x7fff0000u) | e, mn = min_over_frame(key, n);
+            return (key == mn && odd) ? d ^ SGN : d;
+        }
     }
-
-    // Stage n0 (register A, lanes [n0, 2 n0)) to every lane.
-    template <uint32_t n0>
-    __device__ __forceinline__ void lenter() {
-        static_for<0, n0>([&](auto kc) {
-            constexpr uint32_t k = decltype(kc)::value;
-            loc<n0, k>() = __shfl_sync(kFull, A, n0 + k);
-        });
-    }
-
-    template <uint32_t KIND, uint32_t n, uint32_t p>
-    __device__ __forceinline__ void lfg() {
-        constexpr uint32_t h = n / 2;
-        static_for<0, h>([&](auto kc) {
-            constexpr uint32_t k = decltype(kc)::value;
-            const Acc x = loc<n, k>(), y = loc<n, k + h>();
-            Acc r;
-            if constexpr (KIND == OP_F) r = rop_f<T>(x, y);
-            else if constexpr (KIND == OP_G) r = rop_g<T>(x, y, (bw[p / 32] >> ((p % 32) + k)) & 1u);
-            else r = rop_add<T>(x, y);
-            loc<h, k>() = r;
-        });
-    }
-
     template <uint32_t n, uint32_t p>
-    __device__ __forceinline__ uint32_t lhard() {
-        uint32_t b = 0;
-        static_for<0, n>([&](auto kc) {
-            constexpr uint32_t k = decltype(kc)::value;
-            b |= (loc<n, k>() < Acc(0) ? 1u : 0u) << k;
-        });
-        return b;
-    }
-
-    template <uint32_t n, uint32_t p>
-    __device__ __forceinline__ void lr1() { set_field<p / 32, p % 32, n>(lhard<n, p>()); }
-
-    template <uint32_t n, uint32_t p>
-    __device__ __forceinline__ void lrep() {
-        Acc t[n];
-        static_for<0, n>([&](auto kc) { t[decltype(kc)::value] = loc<n, decltype(kc)::value>(); });
-        fold_local<n>(t);
-        set_field<p / 32, p % 32, n>(t[0] < Acc(0) ? kFull : 0u);
-    }
-
-    template <uint32_t n, uint32_t p>
-    __device__ __forceinline__ void lspc() {
-        const uint32_t hd = lhard<n, p>();
-        uint32_t best = mag_bits(loc<n, 0>()), at = 0;
-        static_for<1, n>([&](auto kc) {
-            constexpr uint32_t k = decltype(kc)::value;
-            const uint32_t mg = mag_bits(loc<n, k>());
-            at = mg < best ? k : at;  // strictly smaller: the lowest index keeps a tie
-            best = mg < best ? mg : best;
-        });
-        set_field<p / 32, p % 32, n>(hd ^ ((__popc(hd) & 1u) << at));
+    __device__ __forceinline__ void spc() {
+        if constexpr (n <= G) {
+            if constexpr (n >= E) B[p / E] = spc_small<n>(row<n, 0>());
+            else bits<n, p>() = spc_small<n>(row<n, 0>());
+        } else {
+            constexpr uint32_t K = n / E;
+            uint32_t par = 0;
+            static_for<0, K>([&](auto kc) {
+                constexpr uint32_t k = decltype(kc)::value;
+                const uint32_t d = V::hard(row<n, k>());
+                B[p / E + k] = d;
+                par ^= d;
+            });
+            if constexpr (W == 2) par ^= par << 16;
+            const uint32_t odd = __popc(of_frame<G>(__ballot_sync(kFull, static_cast<int32_t>(par) < 0))) & 1u;
+            if constexpr (W == 1) {
+                uint32_t mk = kFull;
+                static_for<0, K>([&](auto kc) {
+                    mk = min(mk, row<n, decltype(kc)::value>() & 0x7fffffffu);
+                });
+                const uint32_t mn = min_over_frame(mk, G);
+                uint32_t e = kFull;  // lowest index of this lane with that magnitude
+                static_for<0, K>([&](auto kc) {
+                    constexpr uint32_t k = K - 1 - decltype(kc)::value;
+                    if ((row<n, k>() & 0x7fffffffu) == mn) e = E * k + li;
+                });
+                e = min_over_frame(e, G);
+                const uint32_t at = odd ? e - li : kFull;  // E k on the lane that flips row k
+                static_for<0, K>([&](auto kc) {
+                    constexpr uint32_t k = decltype(kc)::value;
+                    if (at == E * k) B[p / E + k] ^= SGN;
+                });
+            } else {
+                uint32_t key = kFull;  // f16 magnitude, then G-chunk, then lane
+                static_for<0, K>([&](auto kc) {
+                    constexpr uint32_t k = decltype(kc)::value;
+                    const uint32_t x = row<n, k>();
+                    key = min(key, ((x << 16) & 0x7fff0000u) | (64u * k));
+                    key = min(key, (x & 0x7fff0000u) | (64u * k + 32u));
+                });
+                key |= li;
+                const uint32_t mn = min_over_frame(key, G);
+                const uint32_t c = (key == mn && odd) ? (mn & 0xffffu) >> 5 : kFull;  // chunk to flip
+                static_for<0, K>([&](auto kc) {
+                    constexpr uint32_t k = decltype(kc)::value;
+                    if (c == 2 * k) B[p / E + k] ^= 0x00008000u;
+                    if (c == 2 * k + 1) B[p / E + k] ^= 0x80000000u;
+                });
+            }
+        }
     }
 
     // Repetition-SPC node of n leaves (8 or 16) at subtree offset p, decoded
     // speculatively (Sec. II-D): F feeds the Repetition child while G for a
     // left estimate of all zeros and for one of all ones feed two SPC decodes;
     // the Repetition decision selects one SPC estimate and Eq. 3 joins the
-    // halves. Bit-identical to F, rep, G, spc, combine in that order (the fold
-    // order of the sum and the SPC tie rule are the ones rep<> and spc<> use).
+    // halves. Bit-identical to F, rep, G, spc, combine in that order.
     template <uint32_t n, uint32_t p>
     __device__ __forceinline__ void repspc() {
-        static_assert(n == 8 || n == 16, "Repetition-SPC node in the shuffle layout");
+        static_assert((n == 8 || n == 16) && n < E, "Repetition-SPC node in the replicated layout");
         constexpr uint32_t h = n / 2;
-        const bool act = lane < h;
-        const Acc x = __shfl_sync(kFull, A, (n + lane) & 31u);      // alpha_v[i], i = lane
-        const Acc y = __shfl_sync(kFull, A, (n + h + lane) & 31u);  // alpha_v[i + h]
-        Acc s = rop_f<T>(x, y);
-#pragma unroll
-        for (uint32_t m = h / 2; m >= 1; m /= 2) {
-            const Acc t = __shfl_down_sync(kFull, s, m);
-            if (lane < m) s = rop_add<T>(s, t);
-        }
-        const bool one = __shfl_sync(kFull, s, 0) < Acc(0);
-        const Acc g0 = rop_g<T>(x, y, 0u), g1 = rop_g<T>(x, y, 1u);
-        const uint32_t hd0 = __ballot_sync(kFull, act && g0 < Acc(0));
-        const uint32_t hd1 = __ballot_sync(kFull, act && g1 < Acc(0));
-        const uint32_t m0 = act ? mag_bits(g0) : kFull, m1 = act ? mag_bits(g1) : kFull;
-        const uint32_t mn0 = __reduce_min_sync(kFull, m0), mn1 = __reduce_min_sync(kFull, m1);
-        const uint32_t f0 = __ffs(__ballot_sync(kFull, act && m0 == mn0)) - 1u;
-        const uint32_t f1 = __ffs(__ballot_sync(kFull, act && m1 == mn1)) - 1u;
-        const uint32_t r0 = hd0 ^ ((__popc(hd0) & 1u) << f0);
-        const uint32_t r1 = hd1 ^ ((__popc(hd1) & 1u) << f1);
-        const uint32_t right = one ? r1 : r0;
-        const uint32_t left = (one ? (1u << h) - 1u : 0u) ^ right;
-        set_field<p / 32, p % 32, n>(left | (right << h));
-    }
-
-    template <uint32_t n, uint32_t p>
-    __device__ __forceinline__ void spc() {
-        if constexpr (n >= 32) {
-            constexpr uint32_t K = n / 32;
-            uint32_t par = 0, mk = kFull;
-            static_for<0, K>([&](auto kc) {
-                constexpr uint32_t k = decltype(kc)::value;
-                const uint32_t hd = __ballot_sync(kFull, reg<n, k>() < Acc(0));
-                bw[p / 32 + k] = hd;
-                par ^= __popc(hd);
-                const uint32_t mg = mag_bits(reg<n, k>());
-                mk = mg < mk ? mg : mk;
-            });
-            const uint32_t mn = __reduce_min_sync(kFull, mk);
-            uint32_t e = kFull;  // lowest element index of this lane with |alpha| == mn
-            static_for<0, K>([&](auto kc) {
-                constexpr uint32_t k = K - 1 - decltype(kc)::value;
-                if (mag_bits(reg<n, k>()) == mn) e = 32 * k + lane;
-            });
-            e = __reduce_min_sync(kFull, e);
-            if (par & 1u) {
-                static_for<0, K>([&](auto kc) {
-                    constexpr uint32_t k = decltype(kc)::value;
-                    if ((e >> 5) == k) bw[p / 32 + k] ^= 1u << (e & 31u);
-                });
-            }
-        } else {
-            const bool in = lane >= n && lane < 2 * n;
-            const uint32_t hd = __ballot_sync(kFull, in && A < Acc(0)) >> n;
-            const uint32_t mag = in ? mag_bits(A) : kFull;
-            const uint32_t mn = __reduce_min_sync(kFull, mag);
-            const uint32_t first = (__ffs(__ballot_sync(kFull, in && mag == mn)) - 1u - n) & 31u;
-            set_field<p / 32, p % 32, n>(hd ^ ((__popc(hd) & 1u) << first));
-        }
+        const uint32_t x = t[clog2(n)], z = partner<n>(x);
+        const uint32_t s = rep_small<h>(V::f(x, z));
+        const uint32_t r0 = spc_small<h>(V::add(x, z));
+        const uint32_t r1 = spc_small<h>(V::add(x ^ mask_a<n>(), z ^ mask_b<n>()));
+        const uint32_t r = static_cast<int32_t>(s) < 0 ? r1 : r0;
+        bits<n, p>() = r ^ (s & mask_a<n>());
     }
 };
 
