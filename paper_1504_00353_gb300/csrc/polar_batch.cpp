@@ -133,10 +133,9 @@ polar_status polar_batch_create_ex(polar_code_t *const *codes, uint32_t n_codes,
             return POLAR_EINVAL;  // create the codes with this device current
         }
         const DeviceState &ds = code->dev[device];
-        const size_t nops = code->ops.size();
-        desc[c].ext_mask = ds.tables + 2 * nops;
-        desc[c].ext_pre = ds.tables + 2 * nops + code->NW;
-        desc[c].ext_wstart = ds.tables + 2 * nops + 2 * code->NW;
+        desc[c].ext_mask = ds.tables + code->at_mask();
+        desc[c].ext_mv = ds.tables;
+        desc[c].ext_start = ds.tables + code->at_start();
         desc[c].N = code->N;
         desc[c].K = code->K;
         desc[c].NW = code->NW;

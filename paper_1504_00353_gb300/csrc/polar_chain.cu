@@ -268,7 +268,6 @@ polar_status polar_encode_systematic_device(const polar_code_t *code, const uint
     DeviceState *ds = nullptr;
     const polar_status st = code_device_state(c, device, &ds);
     if (st != POLAR_OK) return st;
-    const size_t nops = c->ops.size();
     const uint32_t nw = c->N >= 32 ? c->N / 32 : 1;
     const size_t smem = nw * sizeof(uint32_t);  // the frame's N bits: 128 KB at N = 2^20
     if (smem > 48 * 1024) {
@@ -284,7 +283,7 @@ polar_status polar_encode_systematic_device(const polar_code_t *code, const uint
     }
     const int grid = static_cast<int>(std::min<size_t>(n_frames, 152 * 8));
     encode_kernel<<<grid, 256, smem, reinterpret_cast<cudaStream_t>(stream)>>>(
-        info_packed, codeword_packed, ds->tables + 2 * nops, ds->tables + 2 * nops + c->NW, c->N,
+        info_packed, codeword_packed, ds->tables + c->at_mask(), ds->tables + c->at_pre(), c->N,
         c->K, n_frames);
     return status_of(cudaGetLastError());
 }

@@ -45,15 +45,14 @@ polar_status ensure_device(polar_code *c, int device, DeviceState **out) {
     if (device < 0 || static_cast<size_t>(device) >= c->dev.size()) return POLAR_ECUDA;
     DeviceState &s = c->dev[device];
     if (!s.ready) {
-        const size_t nops = c->ops.size();
-        const size_t n = 2 * nops + size_t(c->NW) * 2 + c->KW;
-        std::vector<uint32_t> h(std::max<size_t>(n, 1), 0);
+        std::vector<uint32_t> h(c->table_words(), 0);
         const std::vector<uint32_t> d = c->device_ops();
-        std::copy(d.begin(), d.end(), h.begin());
-        std::copy(c->trace_off.begin(), c->trace_off.end(), h.begin() + nops);
-        std::copy(c->ext_mask.begin(), c->ext_mask.end(), h.begin() + 2 * nops);
-        std::copy(c->ext_pre.begin(), c->ext_pre.end(), h.begin() + 2 * nops + c->NW);
-        std::copy(c->ext_wstart.begin(), c->ext_wstart.end(), h.begin() + 2 * nops + 2 * c->NW);
+        std::copy(c->ext_mv.begin(), c->ext_mv.end(), h.begin());
+        std::copy(d.begin(), d.end(), h.begin() + c->at_ops());
+        std::copy(c->trace_off.begin(), c->trace_off.end(), h.begin() + c->at_trace());
+        std::copy(c->ext_mask.begin(), c->ext_mask.end(), h.begin() + c->at_mask());
+        std::copy(c->ext_pre.begin(), c->ext_pre.end(), h.begin() + c->at_pre());
+        std::copy(c->ext_start.begin(), c->ext_start.end(), h.begin() + c->at_start());
         if (cudaMalloc(&s.status, sizeof(int)) != cudaSuccess) return POLAR_ENOMEM;
         if (cudaMalloc(&s.tables, h.size() * 4) != cudaSuccess) {
             cudaFree(s.status);
@@ -281,12 +280,11 @@ polar_status decode_impl(const polar_code_t *code, const void *llr, bool is_i8,
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
 
     KernelArgs a{};
-    const size_t nops = c->ops.size();
-    a.ops = ds->tables;
-    a.trace_offs = ds->tables + nops;
-    a.ext_mask = ds->tables + 2 * nops;
-    a.ext_pre = ds->tables + 2 * nops + c->NW;
-    a.ext_wstart = ds->tables + 2 * nops + 2 * c->NW;
+    a.ops = ds->tables + c->at_ops();
+    a.trace_offs = ds->tables + c->at_trace();
+    a.ext_mask = ds->tables + c->at_mask();
+    a.ext_mv = ds->tables;
+    a.ext_start = ds->tables + c->at_start();
     a.status = ds->status;
     a.llr = llr;
     a.out = bits_out;
@@ -547,11 +545,11 @@ polar_status polar_decode_noalloc(const polar_code_t *code, const float *llr, ui
     }
     const size_t nops = c->ops.size();
     KernelArgs a{};
-    a.ops = ds->tables;
-    a.trace_offs = ds->tables + nops;
-    a.ext_mask = ds->tables + 2 * nops;
-    a.ext_pre = ds->tables + 2 * nops + c->NW;
-    a.ext_wstart = ds->tables + 2 * nops + 2 * c->NW;
+    a.ops = ds->tables + c->at_ops();
+    a.trace_offs = ds->tables + c->at_trace();
+    a.ext_mask = ds->tables + c->at_mask();
+    a.ext_mv = ds->tables;
+    a.ext_start = ds->tables + c->at_start();
     a.status = ds->status;
     a.llr = llr;
     a.out = bits_out;

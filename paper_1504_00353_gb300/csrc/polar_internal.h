@@ -43,7 +43,7 @@ struct LaunchShape {
 struct DeviceState {
     bool ready = false;
     int *status = nullptr;
-    uint32_t *tables = nullptr;  // ops | trace_offs | ext_mask | ext_pre | ext_wstart
+    uint32_t *tables = nullptr;  // ext_mv | ops | trace_offs | ext_mask | ext_pre | ext_start
 };
 
 struct UserLaunch {
@@ -114,7 +114,7 @@ struct polar_code {
     std::vector<uint32_t> trace_off;      // per op (F/G/G_0R), floats
     size_t trace_len = 0;
     uint32_t NW = 1, KW = 0;
-    std::vector<uint32_t> ext_mask, ext_pre, ext_wstart;
+    std::vector<uint32_t> ext_mask, ext_pre, ext_mv, ext_start;
     polar::UserLaunch user[2];
     std::mutex mu;
     // One slot per device ordinal, sized once so pointers into it stay valid.
@@ -220,15 +220,40 @@ struct polar_code {
             ext_pre[w] = pre;
             pre += static_cast<uint32_t>(__builtin_popcount(ext_mask[w]));
         }
-        ext_wstart.assign(KW, 0);
+        ext_start.assign(KW, 0);
         uint32_t w = 0;
         for (uint32_t u = 0; u < KW; ++u) {
             const uint32_t lo = 32 * u;
             while (w < NW && ext_pre[w] + static_cast<uint32_t>(__builtin_popcount(ext_mask[w])) <= lo)
                 ++w;
-            ext_wstart[u] = w;
+            ext_start[u] = (w << 5) | (lo - ext_pre[w]);
+        }
+        ext_mv.assign(size_t(8) * NW, 0);
+        for (uint32_t v = 0; v < NW; ++v) compress_masks(ext_mask[v], &ext_mv[size_t(8) * v]);
+    }
+
+    // Masks of the five steps that pack the bits selected by m to the bottom
+    // (H. S. Warren, "Hacker's Delight", 7-4): mv[i] marks the bits that step i
+    // moves right by 2^i, those with bit i set in their count of zeros of m below.
+    static void compress_masks(uint32_t m, uint32_t *mv) {
+        uint32_t mk = ~m << 1;
+        for (int i = 0; i < 5; ++i) {
+            uint32_t mp = mk;
+            for (int s = 1; s < 32; s *= 2) mp ^= mp << s;  // parity of the zeros below
+            mv[i] = mp & m;
+            m = (m ^ mv[i]) | (mv[i] >> (1 << i));
+            mk &= ~mp;
         }
     }
+
+    // Word offsets of the parts of DeviceState::tables (ext_mv first: it is read
+    // with 16-byte loads).
+    size_t at_ops() const { return size_t(8) * NW; }
+    size_t at_trace() const { return at_ops() + ops.size(); }
+    size_t at_mask() const { return at_trace() + ops.size(); }
+    size_t at_pre() const { return at_mask() + NW; }
+    size_t at_start() const { return at_pre() + NW; }
+    size_t table_words() const { return at_start() + KW; }
 
     // Packed operation words of the interpreter list (see polar_ops.cuh).
     std::vector<uint32_t> device_ops() const {

@@ -1,0 +1,72 @@
+"""Register subtrees and output packing of the specialised decoders at the sizes
+where they can go wrong, bit for bit against the CPU oracle: subtree sizes on both
+sides of a warp's lanes, LLRs with zeros and ties, and rows whose length is no
+multiple of a word. Every comparison is exact (integers and IEEE operations in the
+oracle's order), so no tolerance enters."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle
+from paper_1504_00353_gb300 import polar
+from tests import _cases
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    torch.cuda.set_device(0)
+
+
+def decode(code, y, i8, out=None):
+    t = torch.from_numpy(np.ascontiguousarray(y)).cuda()
+    got = (polar.polar_decode_i8 if i8 else polar.polar_decode)(code, t, out)
+    torch.cuda.synchronize()
+    polar.polar_code_check(code)
+    return got
+
+
+def llrs(rng, n, N, i8):
+    """Small integers: many zeros and equal magnitudes, and int8 sums that saturate."""
+    y = np.where(rng.random((n, N)) < 0.2, rng.integers(-127, 128, (n, N)), rng.integers(-3, 4, (n, N)))
+    return y.astype(np.int8) if i8 else y.astype(np.float32)
+
+
+@pytest.mark.parametrize("N,K", [(2, 1), (32, 9), (64, 33), (128, 31), (256, 97), (1024, 1000),
+                                 (2048, 40), (4096, 3687)])
+@pytest.mark.parametrize("compiled", [False, True])
+def test_packed_rows(N, K, compiled):
+    """Rows of every length mod 4 at every alignment, sparse and dense information sets."""
+    rng = np.random.default_rng(N + K)
+    mask = _cases.random_mask(rng, N, K)
+    code = polar.polar_code_create(N, K, mask)
+    n, row = 37, (K + 7) // 8
+    y = rng.integers(-127, 128, (n, N)).astype(np.int8)
+    want = oracle.decode_batch(mask, y)
+    if compiled:
+        polar.polar_code_compile(code, True, n)
+    buf = torch.full((n * row + 16,), 0xA5, dtype=torch.uint8, device="cuda")
+    for shift in range(4):  # the row's address mod 4; nothing outside the rows is written
+        buf.fill_(0xA5)
+        decode(code, y, True, buf[shift:shift + n * row])
+        got = buf.cpu().numpy()
+        assert np.array_equal(got[shift:shift + n * row].reshape(n, row), want)
+        assert (got[:shift] == 0xA5).all() and (got[shift + n * row:] == 0xA5).all()
+
+
+@pytest.mark.parametrize("i8", [False, True])
+@pytest.mark.parametrize("N,reg", [(4, 32), (16, 32), (32, 32), (64, 32), (64, 64), (64, 128),
+                                   (512, 512)])
+def test_one_frame_subtrees(N, reg, i8):
+    """One frame per warp, subtrees of fewer, as many and more leaves than lanes."""
+    rng = np.random.default_rng(7 * N + reg)
+    for K in sorted({1, N // 4 + 1, N // 2, N - 1}):
+        mask = _cases.random_mask(rng, N, K)
+        code = polar.polar_code_create(N, K, mask)
+        y = llrs(rng, 65, N, i8)
+        polar.polar_code_compile(code, i8, 65, reg)
+        assert np.array_equal(decode(code, y, i8).cpu().numpy(), oracle.decode_batch(mask, y))
