@@ -134,7 +134,8 @@ polar_status polar_batch_create_ex(polar_code_t *const *codes, uint32_t n_codes,
         }
         const DeviceState &ds = code->dev[device];
         desc[c].ext_mask = ds.tables + code->at_mask();
-        desc[c].ext_mv = ds.tables;
+        desc[c].ext_part = ds.tables;
+        desc[c].n_part = static_cast<uint32_t>(code->ext_part.size() / 8);
         desc[c].ext_start = ds.tables + code->at_start();
         desc[c].N = code->N;
         desc[c].K = code->K;

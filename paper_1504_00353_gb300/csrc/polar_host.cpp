@@ -45,9 +45,9 @@ polar_status ensure_device(polar_code *c, int device, DeviceState **out) {
     if (device < 0 || static_cast<size_t>(device) >= c->dev.size()) return POLAR_ECUDA;
     DeviceState &s = c->dev[device];
     if (!s.ready) {
-        std::vector<uint32_t> h(c->table_words(), 0);
+        std::vector<uint32_t> h(std::max<size_t>(c->table_words(), 1), 0);
         const std::vector<uint32_t> d = c->device_ops();
-        std::copy(c->ext_mv.begin(), c->ext_mv.end(), h.begin());
+        std::copy(c->ext_part.begin(), c->ext_part.end(), h.begin());
         std::copy(d.begin(), d.end(), h.begin() + c->at_ops());
         std::copy(c->trace_off.begin(), c->trace_off.end(), h.begin() + c->at_trace());
         std::copy(c->ext_mask.begin(), c->ext_mask.end(), h.begin() + c->at_mask());
@@ -283,7 +283,8 @@ polar_status decode_impl(const polar_code_t *code, const void *llr, bool is_i8,
     a.ops = ds->tables + c->at_ops();
     a.trace_offs = ds->tables + c->at_trace();
     a.ext_mask = ds->tables + c->at_mask();
-    a.ext_mv = ds->tables;
+    a.ext_part = ds->tables;
+    a.n_part = static_cast<uint32_t>(c->ext_part.size() / 8);
     a.ext_start = ds->tables + c->at_start();
     a.status = ds->status;
     a.llr = llr;
@@ -548,7 +549,8 @@ polar_status polar_decode_noalloc(const polar_code_t *code, const float *llr, ui
     a.ops = ds->tables + c->at_ops();
     a.trace_offs = ds->tables + c->at_trace();
     a.ext_mask = ds->tables + c->at_mask();
-    a.ext_mv = ds->tables;
+    a.ext_part = ds->tables;
+    a.n_part = static_cast<uint32_t>(c->ext_part.size() / 8);
     a.ext_start = ds->tables + c->at_start();
     a.status = ds->status;
     a.llr = llr;

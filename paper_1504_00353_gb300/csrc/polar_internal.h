@@ -43,7 +43,7 @@ struct LaunchShape {
 struct DeviceState {
     bool ready = false;
     int *status = nullptr;
-    uint32_t *tables = nullptr;  // ext_mv | ops | trace_offs | ext_mask | ext_pre | ext_start
+    uint32_t *tables = nullptr;  // ext_part | ops | trace_offs | ext_mask | ext_pre | ext_start
 };
 
 struct UserLaunch {
@@ -114,7 +114,7 @@ struct polar_code {
     std::vector<uint32_t> trace_off;      // per op (F/G/G_0R), floats
     size_t trace_len = 0;
     uint32_t NW = 1, KW = 0;
-    std::vector<uint32_t> ext_mask, ext_pre, ext_mv, ext_start;
+    std::vector<uint32_t> ext_mask, ext_pre, ext_part, ext_start;
     polar::UserLaunch user[2];
     std::mutex mu;
     // One slot per device ordinal, sized once so pointers into it stay valid.
@@ -228,8 +228,13 @@ struct polar_code {
                 ++w;
             ext_start[u] = (w << 5) | (lo - ext_pre[w]);
         }
-        ext_mv.assign(size_t(8) * NW, 0);
-        for (uint32_t v = 0; v < NW; ++v) compress_masks(ext_mask[v], &ext_mv[size_t(8) * v]);
+        ext_part.clear();
+        for (uint32_t v = 0; v < NW; ++v) {
+            if (ext_mask[v] == 0 || ext_mask[v] == ~0u) continue;
+            uint32_t rec[8] = {v, ext_mask[v]};
+            compress_masks(ext_mask[v], rec + 2);
+            ext_part.insert(ext_part.end(), rec, rec + 8);
+        }
     }
 
     // Masks of the five steps that pack the bits selected by m to the bottom
@@ -246,9 +251,9 @@ struct polar_code {
         }
     }
 
-    // Word offsets of the parts of DeviceState::tables (ext_mv first: it is read
-    // with 16-byte loads).
-    size_t at_ops() const { return size_t(8) * NW; }
+    // Word offsets of the parts of DeviceState::tables (ext_part first: it is
+    // read with 16-byte loads).
+    size_t at_ops() const { return ext_part.size(); }
     size_t at_trace() const { return at_ops() + ops.size(); }
     size_t at_mask() const { return at_trace() + ops.size(); }
     size_t at_pre() const { return at_mask() + NW; }

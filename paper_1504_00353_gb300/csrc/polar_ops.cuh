@@ -81,7 +81,8 @@ struct KernelArgs {
     const uint32_t *ops;           // n_ops packed operation words
     const uint32_t *trace_offs;    // per op: offset of its F/G/G_0R outputs in a trace row
     const uint32_t *ext_mask;      // info mask of each beta word (NW words)
-    const uint32_t *ext_mv;        // its five compress masks (8 words per beta word, 16-byte aligned)
+    const uint32_t *ext_part;      // words mixing frozen and info bits: n_part records of 8 words
+                                   // (word, mask, five compress masks, 0), 16-byte aligned
     const uint32_t *ext_start;     // per output word: first beta word << 5 | its info bits to skip
     int *status;                   // error flags (bit 0: a bounded wait expired)
     const void *llr;
@@ -97,6 +98,7 @@ struct KernelArgs {
     uint32_t log2W;                // ops with log2(N_v) <= log2W run on warp 0 alone
     uint32_t NW;                   // beta words (max(1, N/32))
     uint32_t KW;                   // output 32-bit words (ceil(K/32))
+    uint32_t n_part;               // records of ext_part
     uint32_t out_row;              // bytes per output row (ceil(K/8))
 };
 
@@ -105,9 +107,9 @@ __host__ __device__ constexpr size_t align_up(size_t v, size_t a) { return (v + 
 // One code of a mixed batch, as the batch kernel sees it.
 struct CodeDesc {
     const uint32_t *ext_mask;      // as in KernelArgs
-    const uint32_t *ext_mv;
+    const uint32_t *ext_part;
     const uint32_t *ext_start;
-    uint32_t N, K, NW, KW, out_row;
+    uint32_t N, K, NW, KW, out_row, n_part;
     uint32_t S;                    // smem_stage_max of this code (clipped to N/2)
 };
 
@@ -857,46 +859,48 @@ __device__ __forceinline__ void exec_op(uint32_t kind, uint32_t n, uint32_t o, c
 
 // ---------------------------------------------------------------- packed output
 
-// The bits of x selected by m, packed to the bottom: the compress of H. S.
-// Warren, "Hacker's Delight" (7-4), five conditional moves right by 1, 2, 4, 8
-// and 16 with the masks mv[0..4] computed on the host for m. Most words are
-// all information bits (or none) and read no masks.
-__device__ __forceinline__ uint32_t extract(uint32_t x, uint32_t m, const uint32_t *mv) {
-    if (m == kFull || m == 0u) return x & m;
-    const uint4 q = __ldg(reinterpret_cast<const uint4 *>(mv));
-    const uint32_t v[5] = {q.x, q.y, q.z, q.w, __ldg(mv + 4)};
-    x &= m;
-#pragma unroll
-    for (int i = 0; i < 5; ++i) x = (x & ~v[i]) | ((x & v[i]) >> (1 << i));
-    return x;
-}
-
 // Write a frame's information bits: the estimate x_hat (beta) restricted to the
-// information set, packed LSB first into out_row bytes. One lane forms one
-// 32-bit output word u from the beta words it draws on; a warp stores 32 of
-// them at once, as aligned words whatever the row's alignment (the bytes are
-// shifted through the neighbouring lane's word).
-// (A bit-by-bit extract loop took about a fifth of a throughput frame's
-// instructions: (1024, 512) 10,000 float32 frames 45.1 -> 32.9 us,
-// (32768, 29492) 4,096 int8 frames 327 -> 275 us with this form.)
+// information set, packed LSB first into out_row bytes; beta is used up.
+// First the few words that mix frozen and information bits are packed to their
+// bottoms in place: the compress of H. S. Warren, "Hacker's Delight" (7-4), five
+// moves right by 1, 2, 4, 8, 16 with masks the host made once. Then one lane
+// forms one 32-bit output word from the beta words it draws on (two for a dense
+// set), and a warp stores 32 of them as aligned words whatever the row's
+// alignment, the bytes shifted through the neighbouring lane's word.
+// Packing is instruction-bound. A bit-by-bit loop was a fifth of a throughput
+// frame's instructions; with the compress done per output word and lane, where
+// one mixed word made its whole warp wait, it was an eighth. (1024, 512), 10,000
+// float32 frames: 45.1, 32.9, 31.0 us; (32768, 29492), 4,096 int8 frames: 327,
+// 275, 260 us for the three forms.
 template <class Grp, class Tables>
-__device__ __forceinline__ void pack_bits(const uint32_t *beta, const Tables &a, uint8_t *out) {
+__device__ __forceinline__ void pack_bits(uint32_t *beta, const Tables &a, uint8_t *out) {
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t first = Grp::kCta ? (threadIdx.x & ~31u) : 0u;
     const uint32_t step = Grp::kCta ? blockDim.x : 32u;
     const uint32_t sh = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(out)) & 3u;
+    for (uint32_t i = Grp::rank(); i < a.n_part; i += Grp::size()) {
+        const uint4 *rec = reinterpret_cast<const uint4 *>(a.ext_part) + 2 * i;
+        const uint4 p = __ldg(rec), q = __ldg(rec + 1);
+        const uint32_t v[5] = {p.z, p.w, q.x, q.y, q.z};
+        uint32_t x = beta[p.x] & p.y;
+#pragma unroll
+        for (int k = 0; k < 5; ++k) x = (x & ~v[k]) | ((x & v[k]) >> (1 << k));
+        beta[p.x] = x;
+    }
+    Grp::sync();
     for (uint32_t u0 = first; u0 < a.KW; u0 += step) {
         uint32_t acc = 0;
         if (u0 + lane < a.KW) {
             const uint32_t st = __ldg(a.ext_start + u0 + lane);
             uint32_t w = st >> 5;
-            int pos = -static_cast<int>(st & 31u);
-            do {
-                const uint32_t m = __ldg(a.ext_mask + w);
-                const uint32_t e = extract(beta[w], m, a.ext_mv + 8 * size_t(w));
-                acc |= pos >= 0 ? (e << pos) : (e >> -pos);
-                pos += __popc(m);
-            } while (pos < 32 && ++w < a.NW);
+            // the word the output word starts in, without the bits before it
+            uint32_t pos = __popc(__ldg(a.ext_mask + w)) - (st & 31u);
+            acc = beta[w] >> (st & 31u);
+            while (pos < 32 && ++w < a.NW) {
+                const uint32_t c = __popc(__ldg(a.ext_mask + w));
+                if (c) acc |= beta[w] << pos;
+                pos += c;
+            }
         }
         // this lane's aligned word: bytes [4 lane - sh, 4 lane - sh + 4) of the
         // warp's `left` bytes
