@@ -638,9 +638,9 @@ __device__ __forceinline__ void op_r1_f32v(const float *__restrict__ in, uint32_
             const uint32_t i = base + k * step + lane;
             uint32_t b = 0;
             if (i < nv) {
-                const float4 x = v[i];
-                b = (__float_as_uint(x.x) >> 31) | ((__float_as_uint(x.y) >> 30) & 2u) |
-                    ((__float_as_uint(x.z) >> 29) & 4u) | ((__float_as_uint(x.w) >> 28) & 8u);
+                const float4 x = v[i];  // x + 0 has its sign set exactly when x < 0 (-0 decides 0)
+                b = (__float_as_uint(x.x + 0.0f) >> 31) | ((__float_as_uint(x.y + 0.0f) >> 30) & 2u) |
+                    ((__float_as_uint(x.z + 0.0f) >> 29) & 4u) | ((__float_as_uint(x.w + 0.0f) >> 28) & 8u);
             }
             m[k] = b << (4u * (lane & 7u));
         }

@@ -70,3 +70,16 @@ def test_one_frame_subtrees(N, reg, i8):
         y = llrs(rng, 65, N, i8)
         polar.polar_code_compile(code, i8, 65, reg)
         assert np.array_equal(decode(code, y, i8).cpu().numpy(), oracle.decode_batch(mask, y))
+
+
+@pytest.mark.parametrize("compiled", [False, True])
+def test_negative_zero_decides_zero(compiled):
+    """F of a zero and a negative LLR is -0.0, which is not negative: a wide Rate-1 node in
+    memory decides 0 for it."""
+    mask = np.concatenate([np.zeros(512, np.uint8), np.ones(511, np.uint8), [0]]).astype(np.uint8)
+    rng = np.random.default_rng(5)
+    y = rng.integers(-2, 3, (40, 1024)).astype(np.float32)
+    code = polar.polar_code_create(1024, 513, mask)
+    if compiled:
+        polar.polar_code_compile(code, False, 40)
+    assert np.array_equal(decode(code, y, False).cpu().numpy(), oracle.decode_batch(mask, y))
