@@ -206,8 +206,10 @@ polar_status polar_code_set_launch(polar_code_t *code, int is_i8, uint32_t threa
                                    uint32_t smem_stage_max, uint32_t warp_stage_max,
                                    uint32_t ctas_per_sm, uint32_t stage_channel);
 
-/* Several frames per CTA, one per warp (frames = 2, 4 or 8; 0 or 1 = one
- * frame per CTA), for throughput shapes of one warp per frame (threads = 32):
+/* Several frames per CTA, one per warp (frames = 2, 4 or 8; 1 = one frame per
+ * CTA; 0, the default, is the library's choice: four when the launch shape is
+ * left to the library and a decode has at least 12 frames per SM, else one), for
+ * throughput shapes of one warp per frame (threads = 32):
  * the CTA's warps decode different frames side by side with the same
  * straight-line decoder, kept in step by CTA barriers so that they share the
  * instructions they fetch. Applies to the specialised decoder only: compile

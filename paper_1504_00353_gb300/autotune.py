@@ -511,7 +511,7 @@ def configure(code, dtype: str, shape: dict, n_frames: int, interpreter: bool = 
     n_frames frames (unless timing the interpreter)."""
     sh = dict(shape)
     reg = sh.pop("reg_subtree", 0)
-    fpc = sh.pop("frames_per_cta", 1)
+    fpc = sh.pop("frames_per_cta", 1 if sh else 0)  # an empty shape: the library's choice
     local = polar.COMPILE_LOCAL_LEAVES if sh.pop("local_leaves", 0) else 0
     tuned_form = sh.pop("compile_form", "auto")
     if form == "auto":  # an explicit form from the caller wins over the table's

@@ -179,18 +179,41 @@ CompiledKernel *find_compiled(polar_code *c, bool is_i8, const LaunchShape &sh) 
     return it == c->compiled.end() ? nullptr : &it->second;
 }
 
-// The several-frames-per-CTA form of a throughput shape with one warp per
-// frame, when the handle asks for it (polar_code_set_frames_per_cta): F warps,
-// each with its own frame, shared-memory region and scratch; channel read in
-// place. Returns false (sh untouched) when it does not apply.
+// Frames per SM from which the library's own choice for a specialised decoder is
+// several frames per CTA, one per warp. Below, the SMs are not full and a frame
+// is faster with a CTA of its own: 1,280 frames (8 per SM) take the same time or up
+// to 20 % less with one frame per CTA (int8 (2048, 1707) 21.3 vs 21.2 us, (32768,
+// 27000) 134 vs 149), 2,000 and more up to 45 % less with four (25.0 vs 22.8 us;
+// (8192, 6000) 104 vs 74 us for 2,560; (32768, 20000) 447 vs 263 us for 2,000).
+constexpr size_t kMultiFramesPerSm = 12;
+
+// The several-frames-per-CTA form of a throughput shape: F warps, each with its
+// own frame, shared-memory region and scratch; channel read in place. It is the
+// shape of a handle that asks for it (polar_code_set_frames_per_cta, one warp per
+// frame) or that leaves the whole shape to the library. Returns false (sh
+// untouched) when it does not apply.
 bool multi_frame_shape(const polar_code *c, bool is_i8, size_t n_frames, int device,
                        LaunchShape *sh) {
-    const uint32_t F = c->user[is_i8 ? 1 : 0].frames_per_cta;
-    if (F <= 1 || sh->threads != 32) return false;
+    const UserLaunch &u = c->user[is_i8 ? 1 : 0];
     if (n_frames * 2 <= static_cast<size_t>(device_props(device).sms)) return false;  // batch-1 shape
-    const size_t per_frame =
-        (kernel_smem_bytes(c->N, sh->smem_stage_max, 32, is_i8, false) + 127) / 128 * 128;
+    uint32_t F = u.frames_per_cta, S = sh->smem_stage_max;
+    if (F == 0) {
+        if (u.threads || u.smem_stage_max || u.warp_stage_max || u.ctas_per_sm || u.stage_channel)
+            return false;
+        // Four frames; stages up to 1024 LLRs in shared memory (256 to 4096 tried:
+        // within 5 %), 512 for long float32 codes, where the resident frames count
+        // more ((8192, 4500), 4,000 frames: 169 vs 180 us).
+        F = 4;
+        S = std::min<uint32_t>(!is_i8 && c->N >= 8192 ? 512u : 1024u, std::max<uint32_t>(c->N / 2, 1));
+    } else if (F == 1 || sh->threads != 32) {
+        return false;
+    }
+    const uint32_t es = is_i8 ? 1 : 4;
+    const size_t per_frame = (kernel_smem_bytes(c->N, S, 32, is_i8, false) + 127) / 128 * 128;
     if (per_frame * F > device_props(device).smem_optin) return false;
+    const size_t g = (c->N / 2 > S) ? size_t(c->N) - 2 * size_t(S) : 0;
+    sh->smem_stage_max = S;
+    sh->scratch_elems_per_cta = g ? ((g * es + 127) / 128 * 128) / es : 0;
     sh->frames_per_cta = F;
     sh->threads = 32 * F;
     sh->stage_channel = 0;
@@ -198,10 +221,20 @@ bool multi_frame_shape(const polar_code *c, bool is_i8, size_t n_frames, int dev
     return true;
 }
 
-// The specialised decoder for this decode, preferring the several-frames-per-CTA
-// shape when one was compiled for it; *sh becomes the shape of what runs.
+// Whether the library's own choice prefers one frame per CTA for n_frames frames
+// (a handle that asks for several frames per CTA always prefers them).
+bool prefer_one_frame(const polar_code *c, bool is_i8, size_t n_frames, int device) {
+    return c->user[is_i8 ? 1 : 0].frames_per_cta == 0 &&
+           n_frames < kMultiFramesPerSm * static_cast<size_t>(device_props(device).sms);
+}
+
+// The specialised decoder for this decode: of the shapes with one and with several
+// frames per CTA the preferred one if it was compiled, else the other; *sh becomes
+// the shape of what runs.
 CompiledKernel *pick_compiled(polar_code *c, bool is_i8, size_t n_frames, int device,
                               LaunchShape *sh) {
+    CompiledKernel *one = find_compiled(c, is_i8, *sh);
+    if (one && prefer_one_frame(c, is_i8, n_frames, device)) return one;
     LaunchShape msh = *sh;
     if (multi_frame_shape(c, is_i8, n_frames, device, &msh)) {
         if (CompiledKernel *ck = find_compiled(c, is_i8, msh)) {
@@ -209,7 +242,7 @@ CompiledKernel *pick_compiled(polar_code *c, bool is_i8, size_t n_frames, int de
             return ck;
         }
     }
-    return find_compiled(c, is_i8, *sh);
+    return one;
 }
 
 int compiled_occupancy(polar_code *c, CompiledKernel *ck, int device, const LaunchShape &sh) {
@@ -711,7 +744,8 @@ polar_status polar_code_compile_ex(polar_code_t *code, int is_i8, size_t n_frame
     LaunchShape sh{};
     polar_status st = choose_shape(code, is_i8 != 0, n_frames, device, &sh);
     if (st != POLAR_OK) return st;
-    multi_frame_shape(code, is_i8 != 0, n_frames, device, &sh);
+    if (!prefer_one_frame(code, is_i8 != 0, n_frames, device))
+        multi_frame_shape(code, is_i8 != 0, n_frames, device, &sh);
     const uint32_t F = std::max<uint32_t>(sh.frames_per_cta, 1);
     const CompiledKey key{is_i8 != 0, sh.threads, sh.smem_stage_max, sh.warp_stage_max,
                           sh.stage_channel, F};

@@ -83,3 +83,42 @@ def test_negative_zero_decides_zero(compiled):
     if compiled:
         polar.polar_code_compile(code, False, 40)
     assert np.array_equal(decode(code, y, False).cpu().numpy(), oracle.decode_batch(mask, y))
+
+
+@pytest.mark.parametrize("i8", [False, True])
+@pytest.mark.parametrize("N,K", [(2, 1), (8, 3), (64, 33), (512, 257), (2048, 1707), (8192, 4501)])
+def test_library_shape(N, K, i8):
+    """The library's own shape: one frame per CTA for few frames, four for many, and whichever
+    was compiled for decodes of the other size."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    few, many = 4 * sms + 1, 12 * sms + 3
+    rng = np.random.default_rng(N + i8)
+    mask = _cases.random_mask(rng, N, K)
+    y = llrs(rng, many, N, i8)
+    sample = np.unique(np.concatenate([np.arange(3), rng.integers(0, few, 20), [few - 1, many - 1]]))
+    want = oracle.decode_batch(mask, y, frames=sample)
+    for compiled, frames in ((few, 1), (many, 4)):
+        code = polar.polar_code_create(N, K, mask)
+        polar.polar_code_compile(code, i8, compiled)
+        for n in (few, many):
+            assert polar.polar_code_get_launch(code, i8, n)["frames_per_cta"] == frames
+            got = decode(code, y[:n], i8).cpu().numpy()
+            assert np.array_equal(got[sample[sample < n]], want[sample < n]), (compiled, n)
+    both = polar.polar_code_create(N, K, mask)
+    polar.polar_code_compile(both, i8, few)
+    polar.polar_code_compile(both, i8, many)
+    assert polar.polar_code_get_launch(both, i8, few)["frames_per_cta"] == 1
+    assert polar.polar_code_get_launch(both, i8, many)["frames_per_cta"] == 4
+
+
+@pytest.mark.parametrize("i8", [False, True])
+@pytest.mark.parametrize("N", [2, 4, 16, 64, 128, 1024])
+def test_interpreter_subtrees(N, i8):
+    """The interpreter's register subtrees, all node kinds and sides, against the oracle."""
+    rng = np.random.default_rng(3 * N + i8)
+    for K in sorted({1, N // 3 + 1, N // 2, N - N // 8, N - 1}):
+        mask = _cases.random_mask(rng, N, K)
+        y = llrs(rng, 65, N, i8)
+        code = polar.polar_code_create(N, K, mask)
+        assert polar.polar_code_get_launch(code, i8, 65)["unrolled"] == 0
+        assert np.array_equal(decode(code, y, i8).cpu().numpy(), oracle.decode_batch(mask, y))
