@@ -9,12 +9,9 @@
 //     CTA, loads issued ahead of use, one __syncthreads after each;
 //   - narrower operations run on warp 0 alone with __syncwarp between them while
 //     the other warps jump past the run (the host stores the run's end);
-//   - subtrees of at most 32 leaves run entirely in registers of warp 0: every
-//     alpha stage of size 1..16 lives in one register (stage n, element j at
-//     lane n + j), stage 32 in a second one (element j at lane j), and the
-//     subtree's 32 bit estimates in one warp-uniform word. F and G are two
-//     shuffles and one operation, Rate-1 and SPC a ballot (SPC adds a warp min
-//     reduction), Combine is arithmetic on the uniform word.
+//   - subtrees of at most 64 leaves run entirely in registers of warp 0, in the
+//     layout of the specialised decoders (RegSub in polar_ops.cuh), each
+//     operation reached by one jump on its kind, size and side.
 // Memory layout (Sec. III-B): the alpha stage for node size n occupies elements
 // [n, 2n) of a per-CTA array, in shared memory for n <= smem_stage_max and in
 // per-CTA device scratch above that; beta is one N-bit array in shared memory
@@ -50,91 +47,98 @@ __device__ __forceinline__ void trace_store(uint32_t kind, uint32_t n, uint32_t 
 
 // ---------------------------------------------------------------- register subtrees
 
-// A subtree of at most 32 leaves decoded by warp 0 in registers. Stage n <= 16
-// element j is register A on lane n + j; stage 32 element j is register B on
-// lane j; bits[j] of the uniform word `bits` is the estimate of leaf o0 + j.
-template <typename T>
+// A subtree of at most kRegSubtree leaves decoded by warp 0 in registers: the
+// layout and the operations of the specialised decoders (RegSub), reached from
+// the list through one jump on an operation's kind, size and side (whether its
+// node is the right child of its parent), so that an operation is its handful of
+// instructions behind the jump. (Before: shuffles, selects and bit fields with
+// run-time sizes, some 120 instructions for each operation of the list, waiting on
+// one another. 1,000 float32 frames of (1024, 512): 86 -> 80 us.)
+template <typename T, bool TRACE>
 struct RegTree {
-    using Acc = typename Llr<T>::Acc;
-    Acc A, B;
-    uint32_t bits, o0, n0;
+    using Sub = RegSub<T, kRegSubtree, 32, true>;
+    Sub r;
+    uint32_t log2n0, o0;
 
-    __device__ __forceinline__ void enter(const T *src, uint32_t n, uint32_t o, uint32_t lane) {
-        n0 = n;
+    // f(UC<log2 n>{}) for the run-time log2 n <= log2 kRegSubtree.
+    template <uint32_t L = 0, class F>
+    __device__ __forceinline__ static void with_size(uint32_t l, F &&f) {
+        if constexpr ((1u << L) <= kRegSubtree) {
+            if (l == L) f(UC<L>{});
+            else with_size<L + 1>(l, f);
+        }
+    }
+    __device__ __forceinline__ void enter(const T *src, uint32_t l, uint32_t o) {
+        log2n0 = l;
         o0 = o;
-        bits = 0;
-        if (n == 32) {
-            B = static_cast<Acc>(src[lane]);
-        } else {
-            A = (lane >= n && lane < 2 * n) ? static_cast<Acc>(src[lane - n]) : Acc(0);
-        }
+        with_size(l, [&](auto lc) { r.template enter<(1u << decltype(lc)::value)>(src); });
+    }
+    __device__ __forceinline__ void exit(uint32_t *beta) {
+        with_size(log2n0, [&](auto lc) { r.template exit<(1u << decltype(lc)::value)>(beta, o0); });
     }
 
-    __device__ __forceinline__ void set_field(uint32_t p, uint32_t n, uint32_t v) {
-        const uint32_t fm = low_mask(n) << p;
-        bits = (bits & ~fm) | ((v << p) & fm);
-    }
-
-    // Execute one operation of the subtree.
-    __device__ __forceinline__ void exec(uint32_t kind, uint32_t n, uint32_t o, uint32_t lane) {
-        const uint32_t p = o - o0;
-        const Acc src = n == 32 ? B : A;
-        const uint32_t base = n == 32 ? 0u : n;
-        switch (kind) {
-        case OP_F:
-        case OP_G:
-        case OP_G0R: {
-            const uint32_t h = n >> 1;
-            const uint32_t i = lane - h;  // output element of this lane (lanes [h, 2h))
-            const Acc x = __shfl_sync(kFull, src, (base + i) & 31u);
-            const Acc y = __shfl_sync(kFull, src, (base + i + h) & 31u);
-            Acc r;
-            if (kind == OP_F) r = op_f(x, y);
-            else if (kind == OP_G) r = op_g(x, y, (bits >> ((p + i) & 31u)) & 1u);
-            else r = op_add(x, y);
-            if (lane >= h && lane < 2 * h) A = r;
-            break;
-        }
-        case OP_C:
-        case OP_C0R: {
-            const uint32_t h = n >> 1, m = low_mask(h);
-            const uint32_t l = (bits >> p) & m, r = (bits >> (p + h)) & m;
-            set_field(p, h, kind == OP_C ? (l ^ r) : r);
-            break;
-        }
-        case OP_R0: set_field(p, n, 0u); break;
-        case OP_R1: {
-            const bool in = lane >= base && lane < base + n;
-            const uint32_t bal = __ballot_sync(kFull, in && src < Acc(0));
-            set_field(p, n, bal >> base);
-            break;
-        }
-        case OP_REP: {
-            Acc t = src;
-            for (uint32_t m = n >> 1; m > 0; m >>= 1) {
-                const Acc y = __shfl_down_sync(kFull, t, m);
-                if (lane >= base && lane < base + m) t = op_add(t, y);
+    template <uint32_t KIND, uint32_t n>
+    __device__ __forceinline__ void fg(float *row) {
+        r.template fg<KIND, n, 0>();
+        if constexpr (TRACE) {  // the n/2 outputs: value i on lane i
+            const uint32_t lane = threadIdx.x & 31u, v = r.template row<n / 2, 0>();
+            if (lane < n / 2) {
+                if constexpr (sizeof(T) == 1) {
+                    float x;
+                    asm("{\n .reg .b16 l, h;\n mov.b32 {l, h}, %1;\n cvt.f32.f16 %0, l;\n}\n" : "=f"(x) : "r"(v));
+                    row[lane] = x;
+                } else {
+                    row[lane] = __uint_as_float(v);
+                }
             }
-            const Acc s = __shfl_sync(kFull, t, base);
-            set_field(p, n, s < Acc(0) ? kFull : 0u);
-            break;
-        }
-        default: {  // SPC
-            const bool in = lane >= base && lane < base + n;
-            const uint32_t hd = __ballot_sync(kFull, in && src < Acc(0)) >> base;
-            const uint32_t mag = in ? mag_bits(src) : kFull;
-            const uint32_t mn = __reduce_min_sync(kFull, mag);
-            const uint32_t first = __ffs(__ballot_sync(kFull, in && mag == mn)) - 1u - base;
-            set_field(p, n, hd ^ ((__popc(hd) & 1u) << first));
-            break;
-        }
         }
     }
 
-    __device__ __forceinline__ void trace(uint32_t n, uint32_t trace_off, uint32_t lane,
-                                          float *row) const {
-        const uint32_t h = n >> 1;
-        if (lane >= h && lane < 2 * h) row[trace_off + lane - h] = static_cast<float>(A);
+    // Execute the operation of word w; row: where its F/G/G_0R outputs are traced.
+    __device__ __forceinline__ void exec(uint32_t w, float *row) {
+        // a node's bits go to its parent's left or right side; the subtree's root
+        // counts as a left child, and the last operation completes the root
+        const bool inner = !(w & OPW_REG_EXIT);
+        const uint32_t side = inner ? (w >> 12) & 1u : 0u, up = inner ? (w >> 13) & 1u : 0u;
+        // dense keys, so that the switch is a jump table
+        const uint32_t key = (op_log2n(w) * 9u + op_kind(w)) * 2u + (op_kind(w) == OP_R0 ? up : side);
+#define POLAR_KEY(kind, l, s) (((l) * 9u + (kind)) * 2u + (s))
+#define POLAR_FG(l)                                                            \
+    case POLAR_KEY(OP_F, l, 0): case POLAR_KEY(OP_F, l, 1): fg<OP_F, (1u << l)>(row); break;       \
+    case POLAR_KEY(OP_G, l, 0): case POLAR_KEY(OP_G, l, 1): fg<OP_G, (1u << l)>(row); break;       \
+    case POLAR_KEY(OP_G0R, l, 0): case POLAR_KEY(OP_G0R, l, 1): fg<OP_G0R, (1u << l)>(row); break;
+#define POLAR_NODE(l, s)                                                       \
+    case POLAR_KEY(OP_R1, l, s): r.template r1<(1u << l), (s << l)>(); break;      \
+    case POLAR_KEY(OP_REP, l, s): r.template rep<(1u << l), (s << l)>(); break;    \
+    case POLAR_KEY(OP_SPC, l, s): r.template spc<(1u << l), (s << l)>(); break;
+#define POLAR_COMBINE(l, s)                                                    \
+    case POLAR_KEY(OP_C, l, s): r.template combine<(1u << l), (s << l), false>(); break;           \
+    case POLAR_KEY(OP_C0R, l, s): r.template combine<(1u << l), (s << l), true>(); break;
+// a Rate-0 right child of n = 2^l leaves whose parent is on side s
+#define POLAR_R0(l, s) \
+    case POLAR_KEY(OP_R0, l, s): r.template r0_right<(1u << l), ((s << (l + 1)) + (1u << l))>(); break;
+        switch (key) {
+            POLAR_FG(1) POLAR_FG(2) POLAR_FG(3) POLAR_FG(4) POLAR_FG(5) POLAR_FG(6)
+            POLAR_NODE(0, 0) POLAR_NODE(1, 0) POLAR_NODE(2, 0) POLAR_NODE(3, 0) POLAR_NODE(4, 0)
+            POLAR_NODE(5, 0) POLAR_NODE(6, 0) POLAR_NODE(0, 1) POLAR_NODE(1, 1) POLAR_NODE(2, 1)
+            POLAR_NODE(3, 1) POLAR_NODE(4, 1) POLAR_NODE(5, 1)
+            POLAR_COMBINE(1, 0) POLAR_COMBINE(2, 0) POLAR_COMBINE(3, 0) POLAR_COMBINE(4, 0)
+            POLAR_COMBINE(5, 0) POLAR_COMBINE(6, 0) POLAR_COMBINE(1, 1) POLAR_COMBINE(2, 1)
+            POLAR_COMBINE(3, 1) POLAR_COMBINE(4, 1) POLAR_COMBINE(5, 1)
+            POLAR_R0(0, 0) POLAR_R0(1, 0) POLAR_R0(2, 0) POLAR_R0(3, 0) POLAR_R0(4, 0) POLAR_R0(5, 0)
+            POLAR_R0(0, 1) POLAR_R0(1, 1) POLAR_R0(2, 1) POLAR_R0(3, 1) POLAR_R0(4, 1)
+        default: break;
+        }
+#undef POLAR_KEY
+#undef POLAR_FG
+#undef POLAR_NODE
+#undef POLAR_COMBINE
+#undef POLAR_R0
+    }
+
+    // A subtree that is one Rate-0 node.
+    __device__ __forceinline__ void r0_root() {
+        with_size(log2n0, [&](auto lc) { r.template r0<(1u << decltype(lc)::value), 0>(); });
     }
 };
 
@@ -196,21 +200,23 @@ struct InterpBody {
             if (op_log2n(w) <= a.log2W) {
                 // a run of narrow ops: warp 0 executes it, the other warps skip it
                 if (warp == 0) {
-                    RegTree<T> rt;
                     uint32_t j = i;
                     for (;;) {
                         const uint32_t kind = op_kind(w), n = 1u << op_log2n(w), o = op_off(w);
-                        const uint32_t jn = j + 1;
-                        const uint32_t wn = jn < a.n_ops ? win.get(jn) : 0u;
-                        if (w & OPW_REG) {
-                            if (w & OPW_REG_ENTER) rt.enter(fr.stage_in(n), n, o, lane);
-                            rt.exec(kind, n, o, lane);
-                            if (TRACE && kind <= OP_G0R)
-                                rt.trace(n, __ldg(a.trace_offs + j), lane, trace_row);
-                            if (w & OPW_REG_EXIT) {
-                                if (lane == 0) write_field(fr.beta, rt.o0, rt.n0, rt.bits);
-                                __syncwarp();
-                            }
+                        if (w & OPW_REG_ENTER) {  // a register subtree, to its last operation
+                            RegTree<T, TRACE> rt;
+                            rt.enter(fr.stage_in(n), op_log2n(w), o);
+                            if (kind == OP_R0) rt.r0_root();
+                            else
+                                for (;;) {
+                                    const uint32_t x = w & OPW_REG_EXIT ? 0u : win.get(j + 1);
+                                    rt.exec(w, TRACE ? trace_row + __ldg(a.trace_offs + j) : nullptr);
+                                    if (w & OPW_REG_EXIT) break;
+                                    w = x;
+                                    ++j;
+                                }
+                            rt.exit(fr.beta);
+                            __syncwarp();
                         } else {
                             exec_op<T, WarpGrp>(kind, n, o, fr);
                             __syncwarp();
@@ -219,9 +225,9 @@ struct InterpBody {
                                 __syncwarp();
                             }
                         }
-                        j = jn;
-                        if (j >= a.n_ops || op_log2n(wn) > a.log2W) break;
-                        w = wn;
+                        if (++j >= a.n_ops) break;
+                        w = win.get(j);
+                        if (op_log2n(w) > a.log2W) break;
                     }
                     i = j;
                 } else {

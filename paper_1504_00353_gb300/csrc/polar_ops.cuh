@@ -72,8 +72,9 @@ __host__ __device__ inline uint32_t op_kind(uint32_t w) { return w & 0xFu; }
 __host__ __device__ inline uint32_t op_log2n(uint32_t w) { return (w >> 4) & 0x1Fu; }
 __host__ __device__ inline uint32_t op_off(uint32_t w) { return (w >> 12) << op_log2n(w); }
 
-// Largest subtree the interpreter decodes in the registers of one warp.
-constexpr uint32_t kRegSubtree = 32;
+// Largest subtree the interpreter decodes in the registers of one warp: the largest
+// for which a node's side tells where its bits go (two rows of 32 float32 bits).
+constexpr uint32_t kRegSubtree = 64;
 
 // Kernel parameters (identical layout for the interpreter and the generated
 // decoders).
@@ -1274,7 +1275,9 @@ __host__ __device__ constexpr uint32_t clog2(uint32_t v) { return v <= 1 ? 0u : 
 // Measured before and after this layout (int8 unless named): one frame of
 // (32768, 29492) 77.9 -> 67.8 us, 4096 of them 352 -> 327 us (float32 883 -> 829),
 // 2,001 frames of (2048, 1707) 24.6 -> 20.5 us.
-template <typename T, uint32_t R, uint32_t G>
+// LEAN (the interpreter): the masks of operand b are formed when used, five
+// registers fewer for one more logic instruction in a narrow G.
+template <typename T, uint32_t R, uint32_t G, bool LEAN = false>
 struct RegSub {
     using V = SubVal<T>;
     static constexpr uint32_t W = V::W, SGN = V::SGN, E = G * W;
@@ -1329,6 +1332,7 @@ struct RegSub {
     template <uint32_t n>
     __device__ __forceinline__ uint32_t mask_b() {
         if constexpr (W == 2 && n == E) return 0x80000000u;
+        else if constexpr (LEAN) return SGN ^ ca[clog2(n) - 1];
         else return cb[clog2(n) - 1];
     }
     // Bit (lowest value first) mask of a replicated node's n <= G lanes of this frame.
@@ -1338,11 +1342,14 @@ struct RegSub {
         else return (ballot >> gsh) & ((1u << n) - 1u);
     }
     __device__ __forceinline__ uint32_t min_over_frame(uint32_t x, uint32_t n) {
-        if constexpr (G == 32) return __reduce_min_sync(kFull, x);
+        if constexpr (G == 32) {
+            return __reduce_min_sync(kFull, x);
+        } else {
 #pragma unroll
-        for (uint32_t m = G / 2; m >= 1; m /= 2)
-            if (m < n) x = min(x, __shfl_xor_sync(kFull, x, m));
-        return x;
+            for (uint32_t m = G / 2; m >= 1; m /= 2)
+                if (m < n) x = min(x, __shfl_xor_sync(kFull, x, m));
+            return x;
+        }
     }
 
     // Load the subtree root's LLRs (stage n0) of this lane's frame.
