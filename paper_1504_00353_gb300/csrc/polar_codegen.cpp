@@ -220,7 +220,7 @@ std::map<size_t, size_t> emit_subtree_functions(std::ostringstream &o, const std
             it = ids.emplace(key, id).first;
             o << "__device__ __noinline__ void " << prefix << "sub" << id << "(const " << T
               << " *in, uint32_t *beta, uint32_t o0) {\n"
-              << "  RegSub<" << T << ", " << R << "u, 32u> r;\n"
+              << "  RegSub<" << T << ", " << R << "u> r;\n"
               << "  r.template enter<" << n0 << "u>(in);\n" << b.str()
               << "  r.template exit<" << n0 << "u>(beta, o0);\n}\n";
         }
@@ -494,7 +494,7 @@ void emit_body(std::ostringstream &o, const polar_code &code, bool is_i8, uint32
         if (op.flags & OPW_REG_ENTER) {
             o0 = op.off;
             n0 = n;
-            o << "      {\n        RegSub<T, " << R << "u, 32u> r;\n"
+            o << "      {\n        RegSub<T, " << R << "u> r;\n"
               << "        r.template enter<" << n0 << "u>(" << in(n0) << ");\n";
         }
         i += emit_reg_op(o, ops, i, o0, "        ") - 1;

@@ -56,7 +56,7 @@ __device__ __forceinline__ void trace_store(uint32_t kind, uint32_t n, uint32_t 
 // one another. 1,000 float32 frames of (1024, 512): 86 -> 80 us.)
 template <typename T, bool TRACE>
 struct RegTree {
-    using Sub = RegSub<T, kRegSubtree, 32, true>;
+    using Sub = RegSub<T, kRegSubtree, true>;
     Sub r;
     uint32_t log2n0, o0;
 

@@ -223,26 +223,15 @@ __device__ __forceinline__ uint32_t hadd2(uint32_t a, uint32_t b) {
     asm("add.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
     return r;
 }
-__device__ __forceinline__ uint32_t hmin2(uint32_t a, uint32_t b) {
-    uint32_t r;
-    asm("min.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
-    return r;
-}
-__device__ __forceinline__ uint32_t hmax2(uint32_t a, uint32_t b) {
-    uint32_t r;
-    asm("max.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
-    return r;
-}
 // Eq. 1 on two f16 lanes: min(|a|, |b|) carrying the XOR of the signs.
 __device__ __forceinline__ uint32_t hf2(uint32_t a, uint32_t b) {
     uint32_t r;
     asm("min.xorsign.abs.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
     return r;
 }
-// Clamp both f16 lanes to [-127, 127] (0xD7F0 = -127, 0x57F0 = 127).
-__device__ __forceinline__ uint32_t hsat2(uint32_t v) {
-    return hmin2(hmax2(v, 0xD7F0D7F0u), 0x57F057F0u);
-}
+// Clamp both f16 lanes to [-127, 127] in one instruction: Eq. 1 with the constant
+// 127 (0x57F0) is min(|v|, 127) with the sign of v.
+__device__ __forceinline__ uint32_t hsat2(uint32_t v) { return hf2(v, 0x57F057F0u); }
 
 // Four int8 LLRs as two f16x2 words: bytes 0, 1 in lo, bytes 2, 3 in hi.
 struct H4 {
@@ -1248,21 +1237,15 @@ template <> struct SubVal<int8_t> {
     __device__ static __forceinline__ uint32_t hard(uint32_t a) { return hadd2(a, 0u); }
 };
 
-// Unsigned type of G bits (the bits of one chunk of a frame's values).
-template <uint32_t G> struct BetaUnit { using type = uint8_t; };
-template <> struct BetaUnit<16> { using type = unsigned short; };
-
 __host__ __device__ constexpr uint32_t clog2(uint32_t v) { return v <= 1 ? 0u : 1u + clog2(v / 2); }
 
-// Subtree of at most R leaves decoded in registers with compile-time node sizes
-// and offsets (the generated decoders), G lanes per frame: G = 32 is one frame
-// per warp; with G = 8 or 16 one warp decodes the same subtree of 32 / G frames
-// at once, lanes [gG, gG + G) holding frame g.
+// Subtree of at most R leaves decoded by one warp in registers with compile-time
+// node sizes and offsets (the generated decoders).
 //
-// Layout. A row is one register per lane: E = G W values of a node. Value e of
-// a stage of n >= E values sits in row e / E, half (e / G) % W, lane e % G, so F
+// Layout. A row is one register per lane: E = 32 W values of a node. Value e of
+// a stage of n >= E values sits in row e / E, half (e / 32) % W, lane e % 32, so F
 // and G of nodes of 2E and more values are lane-local. At n = E with W = 2 the
-// two operands are the halves of one register. A stage of n <= G values is
+// two operands are the halves of one register. A stage of n <= 32 values is
 // kept replicated: every lane li (and both halves) holds value li % n. Then the
 // partner operand of F and G is one shuffle away (lane li ^ n/2), is kept from F
 // for the G of the same node, no lane idles and none needs a predicate, every
@@ -1277,25 +1260,23 @@ __host__ __device__ constexpr uint32_t clog2(uint32_t v) { return v <= 1 ? 0u : 
 // 2,001 frames of (2048, 1707) 24.6 -> 20.5 us.
 // LEAN (the interpreter): the masks of operand b are formed when used, five
 // registers fewer for one more logic instruction in a narrow G.
-template <typename T, uint32_t R, uint32_t G, bool LEAN = false>
+template <typename T, uint32_t R, bool LEAN = false>
 struct RegSub {
     using V = SubVal<T>;
-    static constexpr uint32_t W = V::W, SGN = V::SGN, E = G * W;
+    static constexpr uint32_t G = 32, W = V::W, SGN = V::SGN, E = G * W;
     static constexpr uint32_t NR = R >= E ? R / E : 1;
     uint32_t v32[32], v16[16], v8[8], v4[4], v2[2], v1;  // stages of n >= E values: n / E rows
     uint32_t t[7], y[7];       // stage 2^k < E (replicated); partner operand of node 2^k <= E
     uint32_t B[NR];            // bits of nodes of n >= E values, by row
     uint32_t bl[7], br[7];     // bits of left / right nodes of 2^k < E values (replicated)
     uint32_t ca[5], cb[5];     // sign mask on lanes with bit k of the lane index clear / set
-    uint32_t li, gsh;          // lane within the frame, first lane of the frame
+    uint32_t li;               // lane
 
     __device__ __forceinline__ void init() {
-        const uint32_t lane = threadIdx.x & 31u;
-        li = lane & (G - 1u);
-        gsh = lane & ~(G - 1u);
+        li = threadIdx.x & 31u;
         static_for<0, 5>([&](auto kc) {
             constexpr uint32_t k = decltype(kc)::value;
-            ca[k] = (lane >> k) & 1u ? 0u : SGN;
+            ca[k] = (li >> k) & 1u ? 0u : SGN;
             cb[k] = SGN ^ ca[k];
         });
     }
@@ -1335,24 +1316,17 @@ struct RegSub {
         else if constexpr (LEAN) return SGN ^ ca[clog2(n) - 1];
         else return cb[clog2(n) - 1];
     }
-    // Bit (lowest value first) mask of a replicated node's n <= G lanes of this frame.
+    // Whether the signs of the n <= 32 values x (replicated) have odd parity, as
+    // sign masks (SGN or 0 in every lane): one copy of the values is XORed over the
+    // warp. (A ballot and a population count before: 20 cycles more in the chain.)
     template <uint32_t n>
-    __device__ __forceinline__ uint32_t of_frame(uint32_t ballot) {
-        if constexpr (G == 32) return n == 32 ? ballot : (ballot & ((1u << n) - 1u));
-        else return (ballot >> gsh) & ((1u << n) - 1u);
-    }
-    __device__ __forceinline__ uint32_t min_over_frame(uint32_t x, uint32_t n) {
-        if constexpr (G == 32) {
-            return __reduce_min_sync(kFull, x);
-        } else {
-#pragma unroll
-            for (uint32_t m = G / 2; m >= 1; m /= 2)
-                if (m < n) x = min(x, __shfl_xor_sync(kFull, x, m));
-            return x;
-        }
+    __device__ __forceinline__ uint32_t odd_signs(uint32_t x) {
+        uint32_t keep = SGN;
+        static_for<clog2(n), 5>([&](auto kc) { keep &= ca[decltype(kc)::value]; });
+        return __reduce_xor_sync(kFull, x & keep);
     }
 
-    // Load the subtree root's LLRs (stage n0) of this lane's frame.
+    // Load the subtree root's LLRs (stage n0).
     template <uint32_t n0>
     __device__ __forceinline__ void enter(const T *src) {
         init();
@@ -1375,30 +1349,22 @@ struct RegSub {
                      0xE480E480u);
     }
 
-    // Store the subtree's n0 bits at leaf offset o0 of this lane's frame's beta.
+    // Store the subtree's n0 bits at leaf offset o0 of beta. The words are the same
+    // on every lane, so lane 0 stores them, 16 bytes at a time (o0 is a multiple of
+    // n0, so the words are 16-byte aligned from 128 leaves up).
     template <uint32_t n0>
     __device__ __forceinline__ void exit(uint32_t *beta, uint32_t o0) {
         if constexpr (n0 < E) {
-            const uint32_t m = of_frame<n0>(__ballot_sync(kFull, (bl[clog2(n0)] & 0x80000000u) != 0u));
-            if (li == 0) {
-                if constexpr (G == 32) {
-                    write_field(beta, o0, n0, m);
-                } else if constexpr (n0 < 8) {
-                    write_field(beta, o0, n0, m);
-                } else {
-                    uint8_t *b = reinterpret_cast<uint8_t *>(beta) + (o0 >> 3);
-                    b[0] = static_cast<uint8_t>(m);
-                    if constexpr (n0 == 16) b[1] = static_cast<uint8_t>(m >> 8);
-                }
-            }
-        } else if constexpr (G == 32) {
+            const uint32_t m = __ballot_sync(kFull, static_cast<int32_t>(bl[clog2(n0)]) < 0);
+            if (li == 0) write_field(beta, o0, n0, m);
+        } else {
             uint32_t w[n0 / 32];
             static_for<0, n0 / 32>([&](auto kc) {
                 constexpr uint32_t k = decltype(kc)::value;
                 constexpr uint32_t m = (W == 2 && k % 2 == 0) ? 0x8000u : 0x80000000u;
                 w[k] = __ballot_sync(kFull, (B[k / W] & m) != 0u);
             });
-            if (li == 0) {  // the words are the same on every lane: 16-byte stores
+            if (li == 0) {
                 static_for<0, n0 / 32>([&](auto kc) {
                     constexpr uint32_t k = decltype(kc)::value;
                     if constexpr (n0 >= 128) {
@@ -1410,25 +1376,9 @@ struct RegSub {
                     }
                 });
             }
-        } else {
-            // chunk k (values [kG, kG + G)) of every frame is one ballot; lane li of
-            // a frame stores chunks li, li + G, ... as G-bit units
-            using U = typename BetaUnit<G>::type;
-            U *b = reinterpret_cast<U *>(beta) + o0 / G;
-            constexpr uint32_t NC = n0 / G, STEP = NC < G ? NC : G;
-            static_for<0, NC / STEP>([&](auto qc) {
-                constexpr uint32_t q = decltype(qc)::value;
-                uint32_t mine = 0;
-                static_for<0, STEP>([&](auto kc) {
-                    constexpr uint32_t k = q * STEP + decltype(kc)::value;
-                    constexpr uint32_t m = (W == 2 && k % 2 == 0) ? 0x8000u : 0x80000000u;
-                    const uint32_t w = __ballot_sync(kFull, (B[k / W] & m) != 0u);
-                    if (li == decltype(kc)::value) mine = w;
-                });
-                if (li < STEP) b[q * STEP + li] = static_cast<U>(mine >> gsh);
-            });
         }
     }
+
     // F / G / G_0R of a node of n leaves at subtree offset p.
     template <uint32_t KIND, uint32_t n, uint32_t p>
     __device__ __forceinline__ void fg() {
@@ -1556,29 +1506,26 @@ struct RegSub {
         }
     }
 
-    // SPC bits of a replicated node of n <= G values x. float32: the least
-    // magnitude over the frame's lanes, then its lowest lane (Listing 2); int8:
-    // magnitude and index fit one key. The flip is a left shift that brings the
-    // chosen value's mask bit to the sign.
+    // SPC bits of a replicated node of n <= 32 values x: the sign of the value of
+    // least magnitude, the lowest index of equals (Listing 2), flips on odd parity.
+    // float32: the least magnitude over the warp, then its lowest lane; the shift
+    // brings that lane's ballot bit to its sign. int8: magnitude and index fit one key.
     template <uint32_t n>
     __device__ __forceinline__ uint32_t spc_small(uint32_t x) {
-        const uint32_t d = V::hard(x), e = li & (n - 1u);
-        const uint32_t odd = __popc(of_frame<n>(__ballot_sync(kFull, static_cast<int32_t>(d) < 0))) & 1u;
+        const uint32_t d = V::hard(x), e = li & (n - 1u), odd = odd_signs<n>(d);
         if constexpr (W == 1) {
-            const uint32_t mag = x & 0x7fffffffu, mn = min_over_frame(mag, n);
-            const uint32_t at = of_frame<n>(__ballot_sync(kFull, mag == mn));
-            const uint32_t pick = at & (0u - at) & (0u - odd);
-            return d ^ ((pick << (31u - e)) & SGN);
+            const uint32_t mag = x & 0x7fffffffu, mn = __reduce_min_sync(kFull, mag);
+            const uint32_t at = __ballot_sync(kFull, mag == mn);
+            return d ^ (((at & (0u - at)) << (31u - e)) & odd);
         } else {
-            const uint32_t key = (x & 0x7fff0000u) | e, mn = min_over_frame(key, n);
-            return (key == mn && odd) ? d ^ SGN : d;
+            const uint32_t key = (x & 0x7fff0000u) | e;
+            return d ^ (key == __reduce_min_sync(kFull, key) ? odd : 0u);
         }
     }
     template <uint32_t n, uint32_t p>
     __device__ __forceinline__ void spc() {
-        if constexpr (n <= G) {
-            if constexpr (n >= E) B[p / E] = spc_small<n>(row<n, 0>());
-            else bits<n, p>() = spc_small<n>(row<n, 0>());
+        if constexpr (n <= 32) {
+            bits<n, p>() = spc_small<n>(row<n, 0>());
         } else {
             constexpr uint32_t K = n / E;
             uint32_t par = 0;
@@ -1589,26 +1536,26 @@ struct RegSub {
                 par ^= d;
             });
             if constexpr (W == 2) par ^= par << 16;
-            const uint32_t odd = __popc(of_frame<G>(__ballot_sync(kFull, static_cast<int32_t>(par) < 0))) & 1u;
+            const bool odd = static_cast<int32_t>(__reduce_xor_sync(kFull, par)) < 0;
             if constexpr (W == 1) {
                 uint32_t mk = kFull;
                 static_for<0, K>([&](auto kc) {
                     mk = min(mk, row<n, decltype(kc)::value>() & 0x7fffffffu);
                 });
-                const uint32_t mn = min_over_frame(mk, G);
+                const uint32_t mn = __reduce_min_sync(kFull, mk);
                 uint32_t e = kFull;  // lowest index of this lane with that magnitude
                 static_for<0, K>([&](auto kc) {
                     constexpr uint32_t k = K - 1 - decltype(kc)::value;
                     if ((row<n, k>() & 0x7fffffffu) == mn) e = E * k + li;
                 });
-                e = min_over_frame(e, G);
+                e = __reduce_min_sync(kFull, e);
                 const uint32_t at = odd ? e - li : kFull;  // E k on the lane that flips row k
                 static_for<0, K>([&](auto kc) {
                     constexpr uint32_t k = decltype(kc)::value;
                     if (at == E * k) B[p / E + k] ^= SGN;
                 });
             } else {
-                uint32_t key = kFull;  // f16 magnitude, then G-chunk, then lane
+                uint32_t key = kFull;  // f16 magnitude, then 32-value chunk, then lane
                 static_for<0, K>([&](auto kc) {
                     constexpr uint32_t k = decltype(kc)::value;
                     const uint32_t x = row<n, k>();
@@ -1616,7 +1563,7 @@ struct RegSub {
                     key = min(key, (x & 0x7fff0000u) | (64u * k + 32u));
                 });
                 key |= li;
-                const uint32_t mn = min_over_frame(key, G);
+                const uint32_t mn = __reduce_min_sync(kFull, key);
                 const uint32_t c = (key == mn && odd) ? (mn & 0xffffu) >> 5 : kFull;  // chunk to flip
                 static_for<0, K>([&](auto kc) {
                     constexpr uint32_t k = decltype(kc)::value;
