@@ -317,6 +317,9 @@ void emit_body(std::ostringstream &o, const polar_code &code, bool is_i8, uint32
         o << indent << "discard_l2<" << grp << ">(gen_in<T, N, S, " << n << "u>(fr), " << n * es
           << "u);\n";
     };
+    // the stage written by an operation on the channel stays in scratch for half
+    // of the tree (see stv)
+    auto far = [&](uint32_t n) { return n == N && scratch(n / 2) ? ", true" : ""; };
     auto rd_name = [](uint32_t rd) {
         return rd == RD_LAST ? "polar::RD_LAST" : (rd == RD_STREAM ? "polar::RD_STREAM" : "polar::RD_NORMAL");
     };
@@ -352,7 +355,7 @@ void emit_body(std::ostringstream &o, const polar_code &code, bool is_i8, uint32
             case OP_F:
             case OP_G:
             case OP_G0R:
-                o << "      mem_fg<T, " << grp << ", " << kind_name(op.kind) << ", " << rd << ">("
+                o << "      mem_fg<T, " << grp << ", " << kind_name(op.kind) << ", " << rd << far(n) << ">("
                   << in(n) << ", " << out(n / 2) << ", " << n / 2 << "u, fr.beta, " << off << "u);\n";
                 break;
             case OP_C:
@@ -380,7 +383,7 @@ void emit_body(std::ostringstream &o, const polar_code &code, bool is_i8, uint32
         case OP_F:
         case OP_G:
         case OP_G0R:
-            o << "      op_fg<T, " << grp << ", " << kind_name(op.kind) << ", " << rd << ">("
+            o << "      op_fg<T, " << grp << ", " << kind_name(op.kind) << ", " << rd << far(n) << ">("
               << in(n) << ", " << out(n / 2) << ", " << n / 2 << "u, fr.beta, " << off << "u);\n";
             break;
         case OP_C:
@@ -441,7 +444,7 @@ void emit_body(std::ostringstream &o, const polar_code &code, bool is_i8, uint32
         o << "      " << (outline_mem ? "mem_chain" : "op_chain") << "<T, " << grp << ", " << len
           << "u, " << kind_name(a.kind) << ", " << kind_name(ops[i + 1].kind) << ", "
           << (len == 3 ? kind_name(ops[i + 2].kind) : "polar::OP_F") << ", " << store << "u, "
-          << rd_name(rd_of(i)) << ">(" << in(n) << ", " << out(n / 2) << ", " << out(n / 4) << ", "
+          << rd_name(rd_of(i)) << far(n) << ">(" << in(n) << ", " << out(n / 2) << ", " << out(n / 4) << ", "
           << (len == 3 ? out(n / 8) : "nullptr") << ", " << n << "u, fr.beta, " << a.off << "u);\n";
     };
 
