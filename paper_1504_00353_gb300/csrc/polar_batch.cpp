@@ -105,7 +105,10 @@ polar_status polar_batch_create_ex(polar_code_t *const *codes, uint32_t n_codes,
     b->threads = threads;
     b->frames_per_cta = warp_frames ? threads / 32 : 1;
     const size_t es = b->elem_bytes();
-    constexpr uint32_t kReg = 256;  // register-resident subtree size of every body
+    // Register-resident subtree of every body: for int8, 512 leaves are eight rows of
+    // f16 pairs (16,384 mixed frames 385 -> 353 us against 256 leaves); for float32
+    // they would be sixteen rows, which crowd the register budget.
+    const uint32_t kReg = is_i8 ? 512 : 256;
     std::vector<CodeDesc> desc(n_codes);
     std::vector<const polar_code *> cc;
     for (uint32_t c = 0; c < n_codes; ++c) {
