@@ -141,35 +141,18 @@ namespace {
 // struct <name> { operator()(frame) }: the code's operation list with every
 // node size and offset written as a constant. S = shared-memory stage cap,
 // W = widest node run on warp 0 alone, R = largest register-resident subtree.
-// ops[i..i+4] are F, Repetition, G, SPC, Combine of one node of 8 or 16 leaves,
-// all inside one register subtree (Sec. II-D, "Repetition-SPC codes").
-bool is_repspc(const std::vector<HostOp> &ops, size_t i) {
-    if (i + 4 >= ops.size()) return false;
-    const HostOp &f = ops[i], &r = ops[i + 1], &g = ops[i + 2], &s = ops[i + 3], &c = ops[i + 4];
-    const uint32_t l = f.log2n;
-    if (f.kind != OP_F || (l != 3 && l != 4)) return false;
-    for (size_t k = i; k <= i + 4; ++k) {
-        if (!(ops[k].flags & OPW_REG)) return false;
-        if (k > i && (ops[k].flags & OPW_REG_ENTER)) return false;
-        if (k < i + 4 && (ops[k].flags & OPW_REG_EXIT)) return false;
-    }
-    return r.kind == OP_REP && r.log2n == l - 1 && r.off == f.off && g.kind == OP_G &&
-           g.log2n == l && g.off == f.off && s.kind == OP_SPC && s.log2n == l - 1 &&
-           s.off == f.off + (1u << (l - 1)) && c.kind == OP_C && c.log2n == l && c.off == f.off;
-}
-
 // The register-subtree operation i (inside a subtree entered at o0 with n0
-// leaves) as a RegSub call; returns the number of list entries it covers: 5 for
-// a fused Repetition-SPC node, 2 for a G whose right child is a Rate-1 node (the
-// child's LLRs are used for their signs only).
+// leaves) as a RegSub call; returns the number of list entries it covers: 2 for a
+// G whose right child is a Rate-1 node (the child's LLRs are used for their signs
+// only). A Repetition-SPC node (Sec. II-D) runs as its five operations: decoding
+// its SPC child for both left estimates at once measured slower, alone on an SM
+// too, since the second SPC costs more instructions than its wait (4,096 int8
+// frames of (32768, 29492) 238 -> 233 us without it, one frame 56.8 -> 56.0,
+// mixed frames 353 -> 340).
 size_t emit_reg_op(std::ostream &o, const std::vector<HostOp> &ops, size_t i, uint32_t o0,
                    const char *indent) {
     const HostOp &op = ops[i];
     const uint32_t n = 1u << op.log2n, p = op.off - o0;
-    if (is_repspc(ops, i)) {  // F, rep, G, spc, combine of one 8- or 16-leaf node
-        o << indent << "r.template repspc<" << n << "u, " << p << "u>();\n";
-        return 5;
-    }
     o << indent << "r.template ";
     if (op.kind == OP_G && ops[i + 1].kind == OP_R1 && ops[i + 1].log2n + 1 == op.log2n) {
         o << "g_r1<" << n << "u, " << p << "u>();\n";

@@ -1588,23 +1588,6 @@ struct RegSub {
             }
         }
     }
-
-    // Repetition-SPC node of n leaves (8 or 16) at subtree offset p, decoded
-    // speculatively (Sec. II-D): F feeds the Repetition child while G for a
-    // left estimate of all zeros and for one of all ones feed two SPC decodes;
-    // the Repetition decision selects one SPC estimate and Eq. 3 joins the
-    // halves. Bit-identical to F, rep, G, spc, combine in that order.
-    template <uint32_t n, uint32_t p>
-    __device__ __forceinline__ void repspc() {
-        static_assert((n == 8 || n == 16) && n < E, "Repetition-SPC node in the replicated layout");
-        constexpr uint32_t h = n / 2;
-        const uint32_t x = t[clog2(n)], z = partner<n>(x);
-        const uint32_t s = rep_small<h>(V::f(x, z));
-        const uint32_t r0 = spc_small<h>(V::add(x, z));
-        const uint32_t r1 = spc_small<h>(V::add(x ^ mask_a<n>(), z ^ mask_b<n>()));
-        const uint32_t r = static_cast<int32_t>(s) < 0 ? r1 : r0;
-        bits<n, p>() = r ^ (s & mask_a<n>());
-    }
 };
 
 // Pointer to stage n of a generated decoder with compile-time N and S.
