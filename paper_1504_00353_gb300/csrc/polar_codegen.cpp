@@ -232,29 +232,6 @@ uint32_t mem_output_stage(const HostOp &op) {
     }
 }
 
-// L2 prefetches: for an operation that reads a stage held in device memory
-// (above S, or the channel when it is read in place), the point where its input
-// is fetched ahead of use is the start of the last register subtree before it,
-// provided no operation in between rewrites that stage (the subtree's work then
-// covers the fetch latency). Returns, per list index, the stages to prefetch
-// there.
-std::vector<std::vector<uint32_t>> plan_prefetch(const std::vector<HostOp> &ops, uint32_t N,
-                                                 uint32_t S, bool chan_global) {
-    std::vector<std::vector<uint32_t>> at(ops.size());
-    for (size_t i = 0; i < ops.size(); ++i) {
-        const uint32_t n = mem_input_stage(ops[i]);
-        if (!n || !((n == N && chan_global) || (n < N && n > S))) continue;
-        for (size_t j = i; j-- > 0;) {
-            if (mem_output_stage(ops[j]) == n) break;  // produced since: still in L2
-            if (ops[j].flags & OPW_REG_ENTER) {
-                at[j].push_back(n);
-                break;
-            }
-        }
-    }
-    return at;
-}
-
 // warp_frames: the body for several frames per CTA, one per warp (run by
 // run_warp_frames): every operation is warp-level on the warp's own frame, and
 // a CTA barrier after each register subtree keeps the warps in step.
@@ -268,7 +245,6 @@ void emit_body(std::ostringstream &o, const polar_code &code, bool is_i8, uint32
     const bool outline_sub = outline & kOutlineSubtrees, outline_mem = outline & kOutlineMemory;
     const uint32_t N = code.N;
     const std::vector<HostOp> ops = code.build_ops(R);
-    const std::vector<std::vector<uint32_t>> prefetch = plan_prefetch(ops, N, S, chan_global);
     const uint32_t es = is_i8 ? 1u : 4u;
     // last[i]: operation i is the last to read its input stage before an
     // operation rewrites it (a register subtree's entry reads its root stage)
@@ -469,8 +445,6 @@ void emit_body(std::ostringstream &o, const polar_code &code, bool is_i8, uint32
             continue;
         }
         const char *align = warp_frames ? "      __syncthreads();\n" : "";
-        for (uint32_t pn : prefetch[i])
-            o << "      prefetch_l2(" << in(pn) << ", " << pn * es << "u);\n";
         if (outline_sub && (op.flags & OPW_REG_ENTER)) {  // the whole subtree is one call
             o << "      " << sub_prefix << "sub" << sub_at.at(i) << "(" << in(n) << ", fr.beta, " << op.off
               << "u);\n      __syncwarp();\n" << align;

@@ -815,19 +815,6 @@ __device__ __forceinline__ void op_rep(const T *in, T *tmp, uint32_t *beta, uint
     }
 }
 
-// ---------------------------------------------------------------- L2 prefetch
-
-// Ask L2 to fetch [p, p + bytes) ahead of use (cp.async.bulk.prefetch: a hint
-// with nothing to wait for). Called by a whole warp; lane k issues the k-th
-// 4 KiB slice. p 16-byte aligned, bytes a multiple of 16.
-__device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes) {
-    for (uint32_t off = (threadIdx.x & 31u) * 4096u; off < bytes; off += 32u * 4096u) {
-        const uint32_t n = bytes - off < 4096u ? bytes - off : 4096u;
-        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;"
-                     ::"l"(static_cast<const char *>(p) + off), "r"(n) : "memory");
-    }
-}
-
 // ---------------------------------------------------------------- frame state
 
 template <typename T>
