@@ -276,9 +276,12 @@ void emit_body(std::ostringstream &o, const polar_code &code, bool is_i8, uint32
         o << indent << "discard_l2<" << grp << ">(gen_in<T, N, S, " << n << "u>(fr), " << n * es
           << "u);\n";
     };
-    // the stage written by an operation on the channel stays in scratch for half
-    // of the tree (see stv)
-    auto far = [&](uint32_t n) { return n == N && scratch(n / 2) ? ", true" : ""; };
+    // how the stage of n values is stored (ST_*): the widest one stays in scratch for
+    // half of the tree, the others are read soon
+    auto st_of = [&](uint32_t n) -> uint32_t {
+        return !scratch(n) ? ST_NORMAL : (n == N / 2 ? ST_FAR : ST_NEAR);
+    };
+    auto wr = [&](uint32_t w) { return w ? ", " + std::to_string(w) + "u" : std::string(); };
     auto rd_name = [](uint32_t rd) {
         return rd == RD_LAST ? "polar::RD_LAST" : (rd == RD_STREAM ? "polar::RD_STREAM" : "polar::RD_NORMAL");
     };
@@ -314,7 +317,7 @@ void emit_body(std::ostringstream &o, const polar_code &code, bool is_i8, uint32
             case OP_F:
             case OP_G:
             case OP_G0R:
-                o << "      mem_fg<T, " << grp << ", " << kind_name(op.kind) << ", " << rd << far(n) << ">("
+                o << "      mem_fg<T, " << grp << ", " << kind_name(op.kind) << ", " << rd << wr(st_of(n / 2)) << ">("
                   << in(n) << ", " << out(n / 2) << ", " << n / 2 << "u, fr.beta, " << off << "u);\n";
                 break;
             case OP_C:
@@ -342,7 +345,7 @@ void emit_body(std::ostringstream &o, const polar_code &code, bool is_i8, uint32
         case OP_F:
         case OP_G:
         case OP_G0R:
-            o << "      op_fg<T, " << grp << ", " << kind_name(op.kind) << ", " << rd << far(n) << ">("
+            o << "      op_fg<T, " << grp << ", " << kind_name(op.kind) << ", " << rd << wr(st_of(n / 2)) << ">("
               << in(n) << ", " << out(n / 2) << ", " << n / 2 << "u, fr.beta, " << off << "u);\n";
             break;
         case OP_C:
@@ -403,8 +406,25 @@ void emit_body(std::ostringstream &o, const polar_code &code, bool is_i8, uint32
         o << "      " << (outline_mem ? "mem_chain" : "op_chain") << "<T, " << grp << ", " << len
           << "u, " << kind_name(a.kind) << ", " << kind_name(ops[i + 1].kind) << ", "
           << (len == 3 ? kind_name(ops[i + 2].kind) : "polar::OP_F") << ", " << store << "u, "
-          << rd_name(rd_of(i)) << far(n) << ">(" << in(n) << ", " << out(n / 2) << ", " << out(n / 4) << ", "
+          << rd_name(rd_of(i))
+          << wr(st_of(n / 2) | st_of(n / 4) << 2 | (len == 3 ? st_of(n / 8) << 4 : 0u)) << ">(" << in(n) << ", " << out(n / 2) << ", " << out(n / 4) << ", "
           << (len == 3 ? out(n / 8) : "nullptr") << ", " << n << "u, fr.beta, " << a.off << "u);\n";
+    };
+
+    // Memory-resident int8 G followed by the Rate-1 decision of its right child: one
+    // op_g_r1. (float32 under its 48-register budget: 702 -> 868 us with it; out of
+    // line it multiplied the compile time of the N = 2^20 decoder.)
+    auto g_r1 = [&](size_t i) {
+        const HostOp &g = ops[i];
+        if (!is_i8 || outline_mem || (g.flags & OPW_REG) || g.kind != OP_G || i + 1 >= ops.size()) return false;
+        const HostOp &r = ops[i + 1];
+        return !(r.flags & OPW_REG) && r.kind == OP_R1 && r.log2n + 1 == g.log2n && r.log2n >= 5 &&
+               r.off == g.off + (1u << r.log2n);
+    };
+    auto g_r1_op = [&](size_t i, const char *grp) {
+        const uint32_t n = 1u << ops[i].log2n;
+        o << "      op_g_r1<" << grp << ", "
+          << rd_name(rd_of(i)) << ">(" << in(n) << ", " << n / 2 << "u, fr.beta, " << ops[i].off << "u);\n";
     };
 
     bool in_run = false;
@@ -420,11 +440,13 @@ void emit_body(std::ostringstream &o, const polar_code &code, bool is_i8, uint32
                 in_run = false;
             }
             o << "    {\n";
+            const bool fused = g_r1(i);
             if (clen > 1) chain_op(i, clen, "CtaGrp");
+            else if (fused) g_r1_op(i, "CtaGrp");
             else mem_op(i, "CtaGrp");
             o << "    }\n    __syncthreads();\n";
             discard(i, "CtaGrp", "    ");
-            i += clen - 1;
+            i += clen - 1 + fused;
             continue;
         }
         if (!in_run) {
@@ -439,9 +461,12 @@ void emit_body(std::ostringstream &o, const polar_code &code, bool is_i8, uint32
             continue;
         }
         if (!(op.flags & OPW_REG)) {
-            mem_op(i, "WarpGrp");
+            const bool fused = g_r1(i);
+            if (fused) g_r1_op(i, "WarpGrp");
+            else mem_op(i, "WarpGrp");
             o << "      __syncwarp();\n";
             discard(i, "WarpGrp", "      ");
+            i += fused;
             continue;
         }
         const char *align = warp_frames ? "      __syncthreads();\n" : "";

@@ -55,6 +55,15 @@ enum OpKind : uint32_t {
 // never written back to DRAM. Hints only: the values read are the same.
 enum : uint32_t { RD_NORMAL = 0, RD_STREAM = 1, RD_LAST = 2 };
 
+// How an operation stores a scratch stage (two bits per output stage): ST_FAR, an
+// L2 evict-first policy, for the widest stage (N/2), which is read again only after
+// a whole half of the tree; ST_NEAR, evict-last, for the narrower ones, which are
+// read soon and discarded after their last read. The frames in flight hold more
+// scratch than L2, beside the streaming channel. (4,096 frames of (32768, 29492):
+// ST_FAR int8 248 -> 238 us, float32 806 -> 786; ST_NEAR int8 223 -> 217, float32
+// unchanged; 16,384 mixed int8 frames 312 -> 288 us.)
+enum : uint32_t { ST_NORMAL = 0, ST_FAR = 1, ST_NEAR = 2 };
+
 // One operation as the interpreter reads it: a 32-bit word
 //   bits 0-3   kind (OpKind)
 //   bits 4-8   log2(N_v)
@@ -251,26 +260,31 @@ __device__ __forceinline__ H4 h4_unpack(uint32_t w) {
 __device__ __forceinline__ uint32_t h4_pack(H4 v) {
     return prmt(hadd2(v.lo, 0x65006500u), hadd2(v.hi, 0x65006500u), 0x6420u);
 }
-// F / G / G_0R on four LLRs; bits4 = beta_l of the four (bit k for element k).
-// G flips the sign of alpha_v[i] where beta_l is 1 (Listing 3's sign XOR): the
-// sign bits of elements 0..3 sit at bits 15, 31 of lo and of hi, and bit k of
-// bits4 reaches them by one multiply (the partial products land on disjoint
-// bits, so nothing carries).
+// beta_l of 16 consecutive values (bit k for value k) as a word from which the sign
+// bits of values 2i and 2i + 1, bits 15 and 31 of an f16 pair, are one shift left by
+// 15 - 2i (a multiply per pair before: 4,096 int8 frames of (32768, 29492) 223 -> 216
+// us, 16,384 mixed frames 312 -> 302 us).
+__device__ __forceinline__ uint32_t spread16(uint32_t bits) { return bits | (bits << 15); }
+// F / G / G_0R on four LLRs, values 4j..4j + 3 of the sixteen of `spread`. G flips
+// the sign of alpha_v[i] where beta_l is 1 (Listing 3's sign XOR).
+__device__ __forceinline__ H4 h4_flip(H4 a, uint32_t spread, uint32_t j) {
+    return {a.lo ^ ((spread << (15u - 4u * j)) & 0x80008000u),
+            a.hi ^ ((spread << (13u - 4u * j)) & 0x80008000u)};
+}
 template <uint32_t KIND>
-__device__ __forceinline__ H4 h4_op(H4 a, H4 b, uint32_t bits4) {
+__device__ __forceinline__ H4 h4_op(H4 a, H4 b, uint32_t spread, uint32_t j) {
     if constexpr (KIND == OP_F) {
         return {hf2(a.lo, b.lo), hf2(a.hi, b.hi)};
     } else if constexpr (KIND == OP_G) {
-        const uint32_t ml = (bits4 * 0x40008000u) & 0x80008000u;
-        const uint32_t mh = (bits4 * 0x10002000u) & 0x80008000u;
-        return {hsat2(hadd2(b.lo, a.lo ^ ml)), hsat2(hadd2(b.hi, a.hi ^ mh))};
+        a = h4_flip(a, spread, j);
+        return {hsat2(hadd2(b.lo, a.lo)), hsat2(hadd2(b.hi, a.hi))};
     } else {
         return {hsat2(hadd2(b.lo, a.lo)), hsat2(hadd2(b.hi, a.hi))};
     }
 }
 template <uint32_t KIND>
-__device__ __forceinline__ uint32_t op_i8x4(uint32_t a, uint32_t b, uint32_t bits4) {
-    return h4_pack(h4_op<KIND>(h4_unpack(a), h4_unpack(b), bits4));
+__device__ __forceinline__ uint32_t op_i8x4(uint32_t a, uint32_t b, uint32_t spread, uint32_t j) {
+    return h4_pack(h4_op<KIND>(h4_unpack(a), h4_unpack(b), spread, j));
 }
 
 // 32-bit word j of a 16-byte vector (j a constant after unrolling).
@@ -335,19 +349,29 @@ __device__ __forceinline__ float4 ldv(const float4 *p, unsigned long long pol) {
         return r;
     }
 }
-// Stores of a stage: FAR = true, an L2 evict-first policy, for the widest scratch
-// stage (N/2), which is read again only after a whole half of the tree: it leaves
-// L2 before the narrower stages, which are read soon. (The frames in flight hold
-// more scratch than L2. Without it: 248 -> 238 us for 4,096 int8 frames of
-// (32768, 29492), 806 -> 786 us float32, 1,532 -> 1,480 us for 64 of N = 2^20.)
-template <bool FAR, class Vec>
-__device__ __forceinline__ void stv(Vec *p, const Vec &v, unsigned long long pol) {
-    if constexpr (!FAR) {
+__device__ __forceinline__ unsigned long long evict_last_policy() {
+    unsigned long long p;
+    asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+struct Policies {  // the policies an operation needs, made once
+    unsigned long long first, last;
+    template <uint32_t RD, uint32_t WR>
+    __device__ __forceinline__ static Policies of() {
+        constexpr bool far = ((WR | (WR >> 2) | (WR >> 4)) & 1u) != 0u;
+        constexpr bool near = ((WR | (WR >> 2) | (WR >> 4)) & 2u) != 0u;
+        return {RD != RD_NORMAL || far ? evict_first_policy() : 0ull, near ? evict_last_policy() : 0ull};
+    }
+};
+template <uint32_t ST, class Vec>
+__device__ __forceinline__ void stv(Vec *p, const Vec &v, const Policies &pol) {
+    if constexpr (ST == ST_NORMAL) {
         *p = v;
     } else {
         const uint4 x = *reinterpret_cast<const uint4 *>(&v);
         asm volatile("st.global.L2::cache_hint.v4.u32 [%0], {%1, %2, %3, %4}, %5;"
-                     ::"l"(p), "r"(x.x), "r"(x.y), "r"(x.z), "r"(x.w), "l"(pol) : "memory");
+                     ::"l"(p), "r"(x.x), "r"(x.y), "r"(x.z), "r"(x.w),
+                     "l"(ST == ST_FAR ? pol.first : pol.last) : "memory");
     }
 }
 __device__ __forceinline__ unsigned long long policy_for(uint32_t rd) {
@@ -422,10 +446,11 @@ __device__ __forceinline__ float4 fg4(float4 a, float4 b, uint32_t bits) {
 template <uint32_t KIND>
 __device__ __forceinline__ uint4 fg4(uint4 a, uint4 b, uint32_t bits) {
     uint4 r;
-    r.x = op_i8x4<KIND>(a.x, b.x, bits & 0xFu);
-    r.y = op_i8x4<KIND>(a.y, b.y, (bits >> 4) & 0xFu);
-    r.z = op_i8x4<KIND>(a.z, b.z, (bits >> 8) & 0xFu);
-    r.w = op_i8x4<KIND>(a.w, b.w, (bits >> 12) & 0xFu);
+    const uint32_t s = spread16(bits);
+    r.x = op_i8x4<KIND>(a.x, b.x, s, 0);
+    r.y = op_i8x4<KIND>(a.y, b.y, s, 1);
+    r.z = op_i8x4<KIND>(a.z, b.z, s, 2);
+    r.w = op_i8x4<KIND>(a.w, b.w, s, 3);
     return r;
 }
 
@@ -439,7 +464,7 @@ __device__ __forceinline__ T fg_scalar(T a, T b, uint32_t bit) {
 // out[i] = op(in[i], in[i + h]) for i < h; in and out never overlap. Four vectors
 // per thread are loaded before any is used, so device-memory operands (the
 // channel at the root, scratch stages) overlap their latency.
-template <typename T, class Grp, uint32_t KIND, uint32_t RD = RD_NORMAL, bool FAR = false>
+template <typename T, class Grp, uint32_t KIND, uint32_t RD = RD_NORMAL, uint32_t WR = 0u>
 __device__ __forceinline__ void op_fg(const T *__restrict__ in, T *__restrict__ out, uint32_t h,
                                       const uint32_t *beta, uint32_t o) {
     using Vec = typename Llr<T>::Vec;
@@ -449,24 +474,24 @@ __device__ __forceinline__ void op_fg(const T *__restrict__ in, T *__restrict__ 
         const Vec *va = reinterpret_cast<const Vec *>(in);
         const Vec *vb = reinterpret_cast<const Vec *>(in + h);
         Vec *vo = reinterpret_cast<Vec *>(out);
-        const unsigned long long pol = policy_for(FAR ? RD_STREAM : RD);
+        const Policies pol = Policies::of<RD, WR>();
         uint32_t v = Grp::rank();
         for (; v + 3 * G < nv; v += 4 * G) {
             Vec a[4], b[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                a[k] = ldv<RD>(va + v + k * G, pol);
-                b[k] = ldv<RD>(vb + v + k * G, pol);
+                a[k] = ldv<RD>(va + v + k * G, pol.first);
+                b[k] = ldv<RD>(vb + v + k * G, pol.first);
             }
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const uint32_t bits = KIND == OP_G ? bits_at(beta, o + (v + k * G) * V, V) : 0u;
-                stv<FAR>(vo + v + k * G, fg4<KIND>(a[k], b[k], bits), pol);
+                stv<WR & 3u>(vo + v + k * G, fg4<KIND>(a[k], b[k], bits), pol);
             }
         }
         for (; v < nv; v += G) {
             const uint32_t bits = KIND == OP_G ? bits_at(beta, o + v * V, V) : 0u;
-            stv<FAR>(vo + v, fg4<KIND>(ldv<RD>(va + v, pol), ldv<RD>(vb + v, pol), bits), pol);
+            stv<WR & 3u>(vo + v, fg4<KIND>(ldv<RD>(va + v, pol.first), ldv<RD>(vb + v, pol.first), bits), pol);
         }
     } else {
         for (uint32_t i = Grp::rank(); i < h; i += Grp::size()) {
@@ -490,7 +515,7 @@ __device__ __forceinline__ void op_fg(const T *__restrict__ in, T *__restrict__ 
 // is always stored): an intermediate stage that no later operation reads is
 // not written at all. RD: how the input stage is read (see RD_LAST).
 template <typename T, class Grp, uint32_t L, uint32_t K0, uint32_t K1, uint32_t K2,
-          uint32_t STORE = 3u, uint32_t RD = RD_NORMAL, bool FAR = false>
+          uint32_t STORE = 3u, uint32_t RD = RD_NORMAL, uint32_t WR = 0u>
 __device__ __forceinline__ void op_chain(const T *__restrict__ in, T *__restrict__ stage1,
                                          T *__restrict__ stage2, T *__restrict__ stage3,
                                          uint32_t n, const uint32_t *beta, uint32_t o) {
@@ -501,18 +526,18 @@ __device__ __forceinline__ void op_chain(const T *__restrict__ in, T *__restrict
     Vec *v1 = reinterpret_cast<Vec *>(stage1);
     Vec *v2 = reinterpret_cast<Vec *>(stage2);
     Vec *v3 = reinterpret_cast<Vec *>(stage3);
-    const unsigned long long pol = policy_for(FAR ? RD_STREAM : RD);
+    const Policies pol = Policies::of<RD, WR>();
     for (uint32_t c = Grp::rank(); c < nvc; c += Grp::size()) {
         Vec x[M];
 #pragma unroll
-        for (uint32_t m = 0; m < M; ++m) x[m] = ldv<RD>(vi + c + m * nvc, pol);
+        for (uint32_t m = 0; m < M; ++m) x[m] = ldv<RD>(vi + c + m * nvc, pol.first);
         if constexpr (sizeof(T) == 1) {
             // int8: word by word in f16 pairs; intermediate stages are packed
             // back to bytes only where they are stored
             uint32_t gb[M / 2];
 #pragma unroll
             for (uint32_t m = 0; m < M / 2; ++m)
-                gb[m] = K0 == OP_G ? bits_at(beta, o + (c + m * nvc) * V, V) : 0u;
+                gb[m] = K0 == OP_G ? spread16(bits_at(beta, o + (c + m * nvc) * V, V)) : 0u;
             Vec y[M / 2], z[M / 4], w;
 #pragma unroll
             for (uint32_t j = 0; j < 4; ++j) {
@@ -521,38 +546,38 @@ __device__ __forceinline__ void op_chain(const T *__restrict__ in, T *__restrict
                 for (uint32_t m = 0; m < M; ++m) xh[m] = h4_unpack(vword(x[m], j));
 #pragma unroll
                 for (uint32_t m = 0; m < M / 2; ++m) {
-                    yh[m] = h4_op<K0>(xh[m], xh[m + M / 2], (gb[m] >> (4 * j)) & 0xFu);
+                    yh[m] = h4_op<K0>(xh[m], xh[m + M / 2], gb[m], j);
                     if (STORE & 1u) set_vword(y[m], j, h4_pack(yh[m]));
                 }
 #pragma unroll
                 for (uint32_t m = 0; m < M / 4; ++m) {
-                    zh[m] = h4_op<K1>(yh[m], yh[m + M / 4], 0u);
+                    zh[m] = h4_op<K1>(yh[m], yh[m + M / 4], 0u, j);
                     if (L == 2 || (STORE & 2u)) set_vword(z[m], j, h4_pack(zh[m]));
                 }
-                if constexpr (L == 3) set_vword(w, j, h4_pack(h4_op<K2>(zh[0], zh[1], 0u)));
+                if constexpr (L == 3) set_vword(w, j, h4_pack(h4_op<K2>(zh[0], zh[1], 0u, j)));
             }
 #pragma unroll
             for (uint32_t m = 0; m < M / 2; ++m)
-                if (STORE & 1u) stv<FAR>(v1 + c + m * nvc, y[m], pol);
+                if (STORE & 1u) stv<WR & 3u>(v1 + c + m * nvc, y[m], pol);
 #pragma unroll
             for (uint32_t m = 0; m < M / 4; ++m)
-                if (L == 2 || (STORE & 2u)) v2[c + m * nvc] = z[m];
-            if constexpr (L == 3) v3[c] = w;
+                if (L == 2 || (STORE & 2u)) stv<(WR >> 2) & 3u>(v2 + c + m * nvc, z[m], pol);
+            if constexpr (L == 3) stv<(WR >> 4) & 3u>(v3 + c, w, pol);
         } else {
             Vec y[M / 2];
 #pragma unroll
             for (uint32_t m = 0; m < M / 2; ++m) {
                 const uint32_t bits = K0 == OP_G ? bits_at(beta, o + (c + m * nvc) * V, V) : 0u;
                 y[m] = fg4<K0>(x[m], x[m + M / 2], bits);
-                if (STORE & 1u) stv<FAR>(v1 + c + m * nvc, y[m], pol);
+                if (STORE & 1u) stv<WR & 3u>(v1 + c + m * nvc, y[m], pol);
             }
             Vec z[M / 4];
 #pragma unroll
             for (uint32_t m = 0; m < M / 4; ++m) {
                 z[m] = fg4<K1>(y[m], y[m + M / 4], 0u);
-                if (L == 2 || (STORE & 2u)) v2[c + m * nvc] = z[m];
+                if (L == 2 || (STORE & 2u)) stv<(WR >> 2) & 3u>(v2 + c + m * nvc, z[m], pol);
             }
-            if constexpr (L == 3) v3[c] = fg4<K2>(z[0], z[1], 0u);
+            if constexpr (L == 3) stv<(WR >> 4) & 3u>(v3 + c, fg4<K2>(z[0], z[1], 0u), pol);
         }
     }
 }
@@ -696,6 +721,59 @@ __device__ __forceinline__ void op_r1(const T *__restrict__ in, uint32_t *beta, 
         const bool neg = idx < n && is_neg(in[idx]);
         const uint32_t bal = __ballot_sync(kFull, neg);
         if (lane == 0) write_field(beta, o + (c << 5), n < 32 ? n : 32, bal);
+    }
+}
+
+// Signs of G on the 16 int8 values of one vector pair, value k at bit k (bits = beta_l).
+// The clamp of the int8 sum keeps its sign, and the sums are never -0 (a byte 0
+// enters as +0).
+__device__ __forceinline__ uint32_t g_signs(uint4 a, uint4 b, uint32_t bits) {
+    uint32_t t = 0;
+    const uint32_t s = spread16(bits);
+#pragma unroll
+    for (uint32_t j = 0; j < 4; ++j) {
+        const H4 x = h4_flip(h4_unpack(vword(a, j)), s, j);
+        const H4 y = h4_unpack(vword(b, j));
+        const uint32_t lo = hadd2(y.lo, x.lo), hi = hadd2(y.hi, x.hi);
+        t |= (((lo >> 15) & 0x00010001u) | ((hi >> 13) & 0x00040004u)) << (4 * j);
+    }
+    return (t | (t >> 15)) & 0xFFFFu;
+}
+// int8 G of node (o, 2h) and the Rate-1 decision of its right child (o + h, h) in one
+// pass, h >= 32: the child's LLRs are only looked at for their signs, so they are
+// neither stored nor read back. In a high-rate code the wide right children are
+// Rate-1 nodes. Loads four vector pairs ahead; two lanes join their bits into a
+// word. (Two operations before: 225 -> 223 us for 4,096 frames of
+// (32768, 29492), mixed frames 316 -> 312.)
+template <class Grp, uint32_t RD = RD_NORMAL>
+__device__ __forceinline__ void op_g_r1(const int8_t *__restrict__ in, uint32_t h, uint32_t *beta,
+                                        uint32_t o) {
+    using Vec = uint4;
+    constexpr uint32_t V = 16, L = 2;
+    const Vec *va = reinterpret_cast<const Vec *>(in);
+    const Vec *vb = reinterpret_cast<const Vec *>(in + h);
+    const uint32_t nv = h / V, lane = threadIdx.x & 31u;
+    const uint32_t w0 = Grp::kCta ? (threadIdx.x & ~31u) : 0u, step = Grp::size();
+    const unsigned long long pol = policy_for(RD);
+    for (uint32_t base = w0; base < nv; base += 4 * step) {
+        Vec a[4], b[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t i = base + k * step + lane;
+            if (i < nv) {
+                a[k] = ldv<RD>(va + i, pol);
+                b[k] = ldv<RD>(vb + i, pol);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t i = base + k * step + lane;
+            uint32_t m = i < nv ? g_signs(a[k], b[k], bits_at(beta, o + i * V, V)) : 0u;
+            m <<= V * (lane & (L - 1u));
+#pragma unroll
+            for (uint32_t x = 1; x < L; x *= 2) m |= __shfl_xor_sync(kFull, m, x);
+            if (i < nv && !(lane & (L - 1u))) beta[((o + h) >> 5) + i / L] = m;
+        }
     }
 }
 
@@ -1070,16 +1148,16 @@ __device__ __forceinline__ void run_warp_frames(const KernelArgs &a, const Body 
 // The memory-resident operations as real calls with run-time sizes: the compact
 // form of a generated decoder uses them so that code size grows with the number
 // of distinct subtrees, not with the length of the operation list.
-template <typename T, class Grp, uint32_t KIND, uint32_t RD = RD_NORMAL, bool FAR = false>
+template <typename T, class Grp, uint32_t KIND, uint32_t RD = RD_NORMAL, uint32_t WR = 0u>
 __device__ __noinline__ void mem_fg(const T *in, T *out, uint32_t h, const uint32_t *beta,
                                     uint32_t o) {
-    op_fg<T, Grp, KIND, RD, FAR>(in, out, h, beta, o);
+    op_fg<T, Grp, KIND, RD, WR>(in, out, h, beta, o);
 }
 template <typename T, class Grp, uint32_t L, uint32_t K0, uint32_t K1, uint32_t K2,
-          uint32_t STORE = 3u, uint32_t RD = RD_NORMAL, bool FAR = false>
+          uint32_t STORE = 3u, uint32_t RD = RD_NORMAL, uint32_t WR = 0u>
 __device__ __noinline__ void mem_chain(const T *in, T *stage1, T *stage2, T *stage3, uint32_t n,
                                        const uint32_t *beta, uint32_t o) {
-    op_chain<T, Grp, L, K0, K1, K2, STORE, RD, FAR>(in, stage1, stage2, stage3, n, beta, o);
+    op_chain<T, Grp, L, K0, K1, K2, STORE, RD, WR>(in, stage1, stage2, stage3, n, beta, o);
 }
 template <class Grp>
 __device__ __noinline__ void mem_combine(uint32_t *beta, uint32_t n, uint32_t o, bool copy) {
