@@ -60,8 +60,8 @@ enum : uint32_t { RD_NORMAL = 0, RD_STREAM = 1, RD_LAST = 2 };
 // a whole half of the tree; ST_NEAR, evict-last, for the narrower ones, which are
 // read soon and discarded after their last read. The frames in flight hold more
 // scratch than L2, beside the streaming channel. (4,096 frames of (32768, 29492):
-// ST_FAR int8 248 -> 238 us, float32 806 -> 786; ST_NEAR int8 223 -> 217, float32
-// unchanged; 16,384 mixed int8 frames 312 -> 288 us.)
+// ST_FAR int8 248 -> 238 us, float32 806 -> 786; ST_NEAR int8 213 -> 206, float32
+// 712 -> 705.)
 enum : uint32_t { ST_NORMAL = 0, ST_FAR = 1, ST_NEAR = 2 };
 
 // One operation as the interpreter reads it: a 32-bit word
@@ -777,12 +777,83 @@ __device__ __forceinline__ void op_g_r1(const int8_t *__restrict__ in, uint32_t 
     }
 }
 
+// SPC on int8 LLRs, n >= 512 (see op_spc): 16 values per lane per 16-byte load, four
+// loads ahead. A vector's least magnitude is a chain of Eq. 1 over its f16 pairs
+// (signs ignored), and its f16 bits above the vector's index make one key, whose
+// minimum over the group names the first vector that holds the node's least
+// magnitude; the value is looked up there at the end. (One value per lane per load
+// before, four loads ahead: a 4,096-value node of a throughput frame waited 32 times
+// for memory: 216 -> 206 us for 4,096 frames of (32768, 29492).)
+template <class Grp>
+__device__ __forceinline__ void op_spc_i8v(const int8_t *__restrict__ in, uint32_t *beta, uint32_t n,
+                                           uint32_t o, unsigned long long *rkey, uint32_t *rpar) {
+    const uint4 *v = reinterpret_cast<const uint4 *>(in);
+    const uint32_t nv = n >> 4, lane = threadIdx.x & 31u;
+    const uint32_t w0 = Grp::kCta ? (threadIdx.x & ~31u) : 0u, step = Grp::size();
+    uint32_t key = kFull, par = 0;
+    for (uint32_t base = w0; base < nv; base += 4 * step) {
+        uint4 x[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (base + k * step + lane < nv) x[k] = v[base + k * step + lane];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t i = base + k * step + lane;
+            uint32_t m = 0;
+            if (i < nv) {
+                m = sign_bits16(x[k]);
+                par ^= m;
+                const H4 p = h4_unpack(x[k].x), q = h4_unpack(x[k].y), r = h4_unpack(x[k].z),
+                         s = h4_unpack(x[k].w);
+                const uint32_t least = hf2(hf2(hf2(p.lo, p.hi), hf2(q.lo, q.hi)),
+                                           hf2(hf2(r.lo, r.hi), hf2(s.lo, s.hi))) & 0x7fff7fffu;
+                key = min(key, (min(least & 0xffffu, least >> 16) << 16) | i);
+            }
+            const uint32_t hi = __shfl_down_sync(kFull, m, 1);
+            if (i < nv && !(lane & 1u)) beta[(o >> 5) + (i >> 1)] = m | (hi << 16);
+        }
+    }
+    key = __reduce_min_sync(kFull, key);
+    par = __reduce_xor_sync(kFull, par);
+    if (Grp::kCta) {
+        const uint32_t w = threadIdx.x >> 5;
+        if (lane == 0) {
+            rkey[w] = key;
+            rpar[w] = par;
+        }
+        Grp::sync();
+        if (w != 0) return;
+        const bool has = lane < (Grp::size() >> 5);
+        key = __reduce_min_sync(kFull, has ? static_cast<uint32_t>(rkey[lane]) : kFull);
+        par = __reduce_xor_sync(kFull, has ? rpar[lane] : 0u);
+    } else {
+        Grp::sync();  // the words written above, before one of them is changed
+    }
+    const uint32_t first = (key & 0xffffu) << 4;
+    const float a = fabsf(static_cast<float>(in[first + (lane & 15u)]));
+    float mag;
+    asm("{\n .reg .b16 h, g;\n mov.b32 {g, h}, %1;\n cvt.f32.f16 %0, h;\n}\n" : "=f"(mag) : "r"(key));
+    const uint32_t at = __ballot_sync(kFull, a == mag);
+    if (lane == 0 && (__popc(par) & 1u)) {
+        const uint32_t pos = o + first + static_cast<uint32_t>(__ffs(static_cast<int>(at))) - 1u;
+        beta[pos >> 5] ^= 1u << (pos & 31u);
+    }
+}
+
 // SPC: hard decisions, their parity, flip the least-|alpha| (lowest index)
 // decision when the parity is odd (Listing 2 returns the first lane equal to
 // the minimum).
-template <typename T, class Grp>
+// VEC = false keeps the one-value form for int8 too (the out-of-line copies: the vector
+// form there multiplies the compile time of a list of thousands of calls).
+template <typename T, class Grp, bool VEC = true>
 __device__ __forceinline__ void op_spc(const T *__restrict__ in, uint32_t *beta, uint32_t n,
                                        uint32_t o, unsigned long long *rkey, uint32_t *rpar) {
+    if constexpr (VEC && sizeof(T) == 1) {
+        if (n >= 512) {
+            op_spc_i8v<Grp>(reinterpret_cast<const int8_t *>(in), beta, n, o, rkey, rpar);
+            return;
+        }
+    }
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t w0 = Grp::kCta ? (threadIdx.x >> 5) : 0u;
     const uint32_t ws = Grp::kCta ? (blockDim.x >> 5) : 1u;
@@ -1178,7 +1249,7 @@ __device__ __noinline__ void mem_rep(const T *in, T *tmp, uint32_t *beta, uint32
 template <typename T, class Grp>
 __device__ __noinline__ void mem_spc(const T *in, uint32_t *beta, uint32_t n, uint32_t o,
                                      unsigned long long *rkey, uint32_t *rpar) {
-    op_spc<T, Grp>(in, beta, n, o, rkey, rpar);
+    op_spc<T, Grp, false>(in, beta, n, o, rkey, rpar);
 }
 
 // ---------------------------------------------------------------- mixed batches

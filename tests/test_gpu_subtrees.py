@@ -122,3 +122,30 @@ def test_interpreter_subtrees(N, i8):
         code = polar.polar_code_create(N, K, mask)
         assert polar.polar_code_get_launch(code, i8, 65)["unrolled"] == 0
         assert np.array_equal(decode(code, y, i8).cpu().numpy(), oracle.decode_batch(mask, y))
+
+
+@pytest.mark.parametrize("threads,F", [(32, 1), (32, 4), (128, 1)])
+@pytest.mark.parametrize("n", [512, 1024, 4096])
+def test_wide_int8_nodes(n, threads, F):
+    """int8 SPC and Rate-1 nodes in memory, the latter right after their G, on one warp and on a
+    CTA: ties of the least magnitude in several vectors, all-zero nodes, odd and even parity."""
+    spc = np.zeros(n, np.uint8)
+    spc[0] = 1
+    for mask in (np.concatenate([spc, np.zeros(n, np.uint8)]), np.concatenate([spc, spc])):
+        N, K = 2 * n, int((mask == 0).sum())
+        rng = np.random.default_rng(n + threads)
+        y = llrs(rng, 150, N, True)
+        y[0] = 0
+        y[1] = 127
+        y[2] = -127
+        y[3:40] = np.where(y[3:40] == 0, 5, y[3:40])
+        code = polar.polar_code_create(N, K, mask)
+        polar.polar_code_set_launch(code, True, threads=threads, smem_stage_max=64 if n < 4096 else 1024,
+                                    warp_stage_max=256 if threads > 32 else 0, stage_channel=2)
+        polar.polar_code_set_frames_per_cta(code, True, F)
+        polar.polar_code_compile(code, True, 150, 256)
+        assert polar.polar_code_get_launch(code, True, 150)["frames_per_cta"] == F
+        want = oracle.decode_batch(mask, y)
+        assert np.array_equal(decode(code, y, True).cpu().numpy(), want)
+        polar.polar_code_compile(code, True, 0)  # and the interpreter
+        assert np.array_equal(decode(code, y, True).cpu().numpy(), want)
