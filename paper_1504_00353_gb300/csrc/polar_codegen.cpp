@@ -277,10 +277,15 @@ void emit_body(std::ostringstream &o, const polar_code &code, bool is_i8, uint32
           << "u);\n";
     };
     // how the stage of n values is stored (ST_*): the widest one stays in scratch for
-    // half of the tree, the others are read soon; a mixed batch, whose short codes
-    // leave L2 room, keeps the plain policy for those (278 vs 284 us)
+    // half of the tree, the others are read soon and discarded after it. A stage of R
+    // values or fewer is read last by a register subtree, which discards nothing, so it
+    // keeps the plain policy: no line is left in L2 with the evict-last priority. So do
+    // the narrower stages of a mixed batch (shared_subs), measured for the five mixed
+    // codes: 278 us for 16,384 frames, 284 with evict-last.
     auto st_of = [&](uint32_t n) -> uint32_t {
-        return !scratch(n) ? ST_NORMAL : (n == N / 2 ? ST_FAR : (shared_subs ? ST_NORMAL : ST_NEAR));
+        if (!scratch(n)) return ST_NORMAL;
+        if (n == N / 2) return ST_FAR;
+        return shared_subs || n <= R ? ST_NORMAL : ST_NEAR;
     };
     auto wr = [&](uint32_t w) { return w ? ", " + std::to_string(w) + "u" : std::string(); };
     auto rd_name = [](uint32_t rd) {
