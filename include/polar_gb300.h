@@ -206,15 +206,16 @@ polar_status polar_code_set_launch(polar_code_t *code, int is_i8, uint32_t threa
                                    uint32_t smem_stage_max, uint32_t warp_stage_max,
                                    uint32_t ctas_per_sm, uint32_t stage_channel);
 
-/* Several frames per CTA, one per warp (frames = 2, 4 or 8; 1 = one frame per
- * CTA; 0, the default, is the library's choice: four when the launch shape is
- * left to the library and a decode has at least 12 frames per SM, else one), for
- * throughput shapes of one warp per frame (threads = 32):
+/* Several frames per CTA, one per warp (frames = 2, 4 or 8; 0 or 1 = one
+ * frame per CTA), for throughput shapes of one warp per frame (threads = 32):
  * the CTA's warps decode different frames side by side with the same
  * straight-line decoder, kept in step by CTA barriers so that they share the
  * instructions they fetch. Applies to the specialised decoder only: compile
  * after setting it (polar_code_compile); decodes whose shape has no such
  * decoder, batch-1 shapes and the interpreter keep one frame per CTA.
+ * A handle on which it was never called leaves the choice to the library: four
+ * frames when its whole launch shape is left to the library too and a decode
+ * has at least 12 frames per SM, else one.
  * Not thread-safe against concurrent decodes of the same handle. */
 polar_status polar_code_set_frames_per_cta(polar_code_t *code, int is_i8, uint32_t frames);
 

@@ -511,13 +511,16 @@ def configure(code, dtype: str, shape: dict, n_frames: int, interpreter: bool = 
     n_frames frames (unless timing the interpreter)."""
     sh = dict(shape)
     reg = sh.pop("reg_subtree", 0)
-    fpc = sh.pop("frames_per_cta", 1 if sh else 0)  # an empty shape: the library's choice
+    # an empty shape leaves the frames per CTA of a handle as they are: the library's choice
+    # unless the program has set them
+    fpc = sh.pop("frames_per_cta", 1 if sh else None)
     local = polar.COMPILE_LOCAL_LEAVES if sh.pop("local_leaves", 0) else 0
     tuned_form = sh.pop("compile_form", "auto")
     if form == "auto":  # an explicit form from the caller wins over the table's
         form = tuned_form
     polar.polar_code_set_launch(code, dtype == "i8", **sh)
-    polar.polar_code_set_frames_per_cta(code, dtype == "i8", fpc)
+    if fpc is not None:
+        polar.polar_code_set_frames_per_cta(code, dtype == "i8", fpc)
     if not interpreter:
         polar.polar_code_compile(code, dtype == "i8", n_frames, reg, COMPILE_FORM[form] | local)
 

@@ -686,7 +686,7 @@ polar_status polar_code_get_launch(const polar_code_t *code, int is_i8, size_t n
 polar_status polar_code_set_frames_per_cta(polar_code_t *code, int is_i8, uint32_t frames) {
     if (!code || frames > 8 || (frames > 1 && !is_pow2(frames))) return POLAR_EINVAL;
     std::lock_guard<std::mutex> g(code->mu);
-    code->user[is_i8 ? 1 : 0].frames_per_cta = frames;
+    code->user[is_i8 ? 1 : 0].frames_per_cta = std::max<uint32_t>(frames, 1);
     return POLAR_OK;
 }
 

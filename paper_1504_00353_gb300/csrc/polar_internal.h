@@ -48,7 +48,8 @@ struct DeviceState {
 
 struct UserLaunch {
     uint32_t threads = 0, smem_stage_max = 0, warp_stage_max = 0, ctas_per_sm = 0,
-             stage_channel = 0, frames_per_cta = 0;
+             stage_channel = 0;
+    uint32_t frames_per_cta = 0;  // 0: never set, the library's choice
 };
 
 // A decoder specialised to one code and launch shape (generated CUDA source

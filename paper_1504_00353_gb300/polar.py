@@ -318,9 +318,9 @@ def polar_code_get_launch(code: PolarCode, is_i8: bool, n_frames: int) -> dict:
 
 
 def polar_code_set_frames_per_cta(code: PolarCode, is_i8: bool, frames: int):
-    """Several frames per CTA, one per warp (2, 4, 8; 1 = one; 0 = the library's
-    choice, the default), for the specialised decoder of one-warp-per-frame shapes
-    (compile afterwards)."""
+    """Several frames per CTA, one per warp (2, 4, 8; 0/1 = one), for the
+    specialised decoder of one-warp-per-frame shapes (compile afterwards). Never
+    called: the library's choice."""
     _check(_lib.polar_code_set_frames_per_cta(code.handle, int(bool(is_i8)), frames),
            "polar_code_set_frames_per_cta")
 

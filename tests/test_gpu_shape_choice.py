@@ -1,0 +1,63 @@
+"""Which decoder a handle runs for a batch size: what a program asked for stays what it gets,
+and every choice gives the oracle's bits."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle
+from paper_1504_00353_gb300 import autotune, polar
+from tests import _cases
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    torch.cuda.set_device(0)
+
+
+def sms():
+    return torch.cuda.get_device_properties(0).multi_processor_count
+
+
+def make(N, K, n, i8, seed=3):
+    rng = np.random.default_rng(seed)
+    mask = _cases.random_mask(rng, N, K)
+    y = rng.integers(-127, 128, (n, N)).astype(np.int8) if i8 else \
+        (rng.standard_normal((n, N)) * 3).astype(np.float32)
+    return mask, y, torch.from_numpy(y).cuda()
+
+
+def check_bits(code, mask, y, t, i8, n):
+    got = (polar.polar_decode_i8 if i8 else polar.polar_decode)(code, t[:n]).cpu().numpy()
+    polar.polar_code_check(code)
+    sample = np.unique(np.concatenate([np.arange(min(3, n)), [n // 2, n - 1]]))
+    assert np.array_equal(got[sample], oracle.decode_batch(mask, y, frames=sample))
+
+
+@pytest.mark.parametrize("i8", [False, True])
+@pytest.mark.parametrize("frames", [0, 1])
+def test_zero_or_one_is_one_frame_per_cta(frames, i8):
+    """polar_code_set_frames_per_cta(0) and (1) both mean one frame per CTA, also for batches
+    for which the library would choose several."""
+    n = 12 * sms() + 3
+    mask, y, t = make(256, 100, n, i8)
+    code = polar.polar_code_create(256, 100, mask)
+    polar.polar_code_set_frames_per_cta(code, i8, frames)
+    polar.polar_code_compile(code, i8, n)
+    launch = polar.polar_code_get_launch(code, i8, n)
+    assert launch["unrolled"] and launch["frames_per_cta"] == 1
+    check_bits(code, mask, y, t, i8, n)
+    autotune.configure(code, "i8" if i8 else "f32", {}, n)  # an empty shape does not undo it
+    assert polar.polar_code_get_launch(code, i8, n)["frames_per_cta"] == 1
+
+
+def test_empty_shape_leaves_the_choice_to_the_library():
+    n = 12 * sms() + 3
+    mask, _, _ = make(256, 100, 1, True)
+    code = polar.polar_code_create(256, 100, mask)
+    autotune.configure(code, "i8", {}, n)
+    assert polar.polar_code_get_launch(code, True, n)["frames_per_cta"] == 4
