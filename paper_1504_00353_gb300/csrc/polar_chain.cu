@@ -179,7 +179,7 @@ __device__ inline void transform_parts(const uint32_t *xs, uint32_t warps, uint3
 // (records `part`, see KernelArgs::ext_part) are spread by the expand of
 // "Hacker's Delight" (7-5), the packing steps undone in reverse. Bound by its
 // instructions and, for short codes, by launch width: one warp per frame up to
-// N = 8192, so a block of 128 threads encodes four (a block per frame with every
+// N = 4096, so a block of 128 threads encodes four (a block per frame with every
 // stage in shared memory: 74 us for 16,384 frames of N = 1024, 35 us for 1,024
 // of N = 32768; now 13 and 17).
 template <uint32_t P>
@@ -416,11 +416,16 @@ polar_status polar_encode_systematic_device(const polar_code_t *code, const uint
     DeviceState *ds = nullptr;
     const polar_status st = code_device_state(c, device, &ds);
     if (st != POLAR_OK) return st;
-    // words per lane and warps per frame: one warp up to N = 8192, then warps
-    // up to eight, then both (the stages across warps need warps <= words)
+    // words per lane and warps per frame: one warp of up to four words up to
+    // N = 4096, then up to four warps, then both (the stages across warps need
+    // warps <= words). More words on fewer warps only lengthen a frame's chain:
+    // with eight words before a second warp 100 frames of N = 8192 and 16384 took
+    // 10.3 us instead of 6.2, 5,000 took 16.4 and 26.6 instead of 14.3 and 20.5;
+    // with two words N = 8192 and more are the same, 20,000 frames of N = 4096
+    // 26.7 instead of 22.5.
     const uint32_t nw = c->N >= 32 ? c->N / 32 : 1;
     uint32_t P = 1, warps = 1;
-    while (32 * P < nw && P < 8) P *= 2;
+    while (32 * P < nw && P < 4) P *= 2;
     while (32 * P * warps < nw) {
         if (warps < P) warps *= 2;
         else P *= 2;
