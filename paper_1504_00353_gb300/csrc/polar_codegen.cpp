@@ -418,19 +418,26 @@ void emit_body(std::ostringstream &o, const polar_code &code, bool is_i8, uint32
     };
 
     // Memory-resident int8 G followed by the Rate-1 decision of its right child: one
-    // op_g_r1. (float32 under its 48-register budget: 702 -> 868 us with it; out of
-    // line it multiplied the compile time of the N = 2^20 decoder.)
+    // op_g_r1, where several frames share a CTA's instructions. One frame per CTA is
+    // faster with the two operations: the eight vectors that op_g_r1 holds do not fit
+    // its small register budgets, and its code is not shared ((32768, 29492) at 64
+    // threads per frame and 32 registers, 1,000 frames: 128 us, 233 with it; at one
+    // warp and 72 registers 147, 200). Four frames per CTA, 4,096 frames: 206 us, 202
+    // with it, 16,384 mixed frames 283, 275. (float32 under its 48-register budget:
+    // 702 -> 868 us with it; out of line it multiplied the compile time of the
+    // N = 2^20 decoder.)
     auto g_r1 = [&](size_t i) {
         const HostOp &g = ops[i];
-        if (!is_i8 || outline_mem || (g.flags & OPW_REG) || g.kind != OP_G || i + 1 >= ops.size()) return false;
+        if (!is_i8 || !warp_frames || outline_mem || (g.flags & OPW_REG) || g.kind != OP_G || i + 1 >= ops.size())
+            return false;
         const HostOp &r = ops[i + 1];
         return !(r.flags & OPW_REG) && r.kind == OP_R1 && r.log2n + 1 == g.log2n && r.log2n >= 5 &&
                r.off == g.off + (1u << r.log2n);
     };
-    auto g_r1_op = [&](size_t i, const char *grp) {
+    auto g_r1_op = [&](size_t i) {
         const uint32_t n = 1u << ops[i].log2n;
-        o << "      op_g_r1<" << grp << ", "
-          << rd_name(rd_of(i)) << ">(" << in(n) << ", " << n / 2 << "u, fr.beta, " << ops[i].off << "u);\n";
+        o << "      op_g_r1<" << rd_name(rd_of(i)) << ">(" << in(n) << ", " << n / 2 << "u, fr.beta, "
+          << ops[i].off << "u);\n";
     };
 
     bool in_run = false;
@@ -446,13 +453,11 @@ void emit_body(std::ostringstream &o, const polar_code &code, bool is_i8, uint32
                 in_run = false;
             }
             o << "    {\n";
-            const bool fused = g_r1(i);
             if (clen > 1) chain_op(i, clen, "CtaGrp");
-            else if (fused) g_r1_op(i, "CtaGrp");
             else mem_op(i, "CtaGrp");
             o << "    }\n    __syncthreads();\n";
             discard(i, "CtaGrp", "    ");
-            i += clen - 1 + fused;
+            i += clen - 1;
             continue;
         }
         if (!in_run) {
@@ -468,7 +473,7 @@ void emit_body(std::ostringstream &o, const polar_code &code, bool is_i8, uint32
         }
         if (!(op.flags & OPW_REG)) {
             const bool fused = g_r1(i);
-            if (fused) g_r1_op(i, "WarpGrp");
+            if (fused) g_r1_op(i);
             else mem_op(i, "WarpGrp");
             o << "      __syncwarp();\n";
             discard(i, "WarpGrp", "      ");

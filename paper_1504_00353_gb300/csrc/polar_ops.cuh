@@ -740,12 +740,12 @@ __device__ __forceinline__ uint32_t g_signs(uint4 a, uint4 b, uint32_t bits) {
     return (t | (t >> 15)) & 0xFFFFu;
 }
 // int8 G of node (o, 2h) and the Rate-1 decision of its right child (o + h, h) in one
-// pass, h >= 32: the child's LLRs are only looked at for their signs, so they are
-// neither stored nor read back. In a high-rate code the wide right children are
-// Rate-1 nodes. Loads four vector pairs ahead; two lanes join their bits into a
-// word. (Two operations before: 225 -> 223 us for 4,096 frames of
-// (32768, 29492), mixed frames 316 -> 312.)
-template <class Grp, uint32_t RD = RD_NORMAL>
+// pass of a warp, h >= 32: the child's LLRs are only looked at for their signs, so
+// they are neither stored nor read back. In a high-rate code the wide right children
+// are Rate-1 nodes. Loads four vector pairs ahead; two lanes join their bits into a
+// word. For several frames per CTA (the generator says why): two operations instead,
+// 206 us, now 202 for 4,096 frames of (32768, 29492), 16,384 mixed frames 283, now 275.
+template <uint32_t RD = RD_NORMAL>
 __device__ __forceinline__ void op_g_r1(const int8_t *__restrict__ in, uint32_t h, uint32_t *beta,
                                         uint32_t o) {
     using Vec = uint4;
@@ -753,21 +753,20 @@ __device__ __forceinline__ void op_g_r1(const int8_t *__restrict__ in, uint32_t 
     const Vec *va = reinterpret_cast<const Vec *>(in);
     const Vec *vb = reinterpret_cast<const Vec *>(in + h);
     const uint32_t nv = h / V, lane = threadIdx.x & 31u;
-    const uint32_t w0 = Grp::kCta ? (threadIdx.x & ~31u) : 0u, step = Grp::size();
     const unsigned long long pol = policy_for(RD);
-    for (uint32_t base = w0; base < nv; base += 4 * step) {
+    for (uint32_t base = 0; base < nv; base += 4 * 32u) {
         Vec a[4], b[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const uint32_t i = base + k * step + lane;
+        for (uint32_t k = 0; k < 4; ++k) {
+            const uint32_t i = base + 32u * k + lane;
             if (i < nv) {
                 a[k] = ldv<RD>(va + i, pol);
                 b[k] = ldv<RD>(vb + i, pol);
             }
         }
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const uint32_t i = base + k * step + lane;
+        for (uint32_t k = 0; k < 4; ++k) {
+            const uint32_t i = base + 32u * k + lane;
             uint32_t m = i < nv ? g_signs(a[k], b[k], bits_at(beta, o + i * V, V)) : 0u;
             m <<= V * (lane & (L - 1u));
 #pragma unroll
