@@ -842,8 +842,10 @@ __device__ __forceinline__ void op_spc_i8v(const int8_t *__restrict__ in, uint32
 // SPC: hard decisions, their parity, flip the least-|alpha| (lowest index)
 // decision when the parity is odd (Listing 2 returns the first lane equal to
 // the minimum).
-// VEC = false keeps the one-value form for int8 too (the out-of-line copies: the vector
-// form there multiplies the compile time of a list of thousands of calls).
+// VEC = false keeps the one-value form for int8 too: in the out-of-line copies, where the
+// vector form multiplies the compile time of a list of thousands of calls, and in the
+// interpreter, whose 64 registers its four vectors overrun (208 bytes of spills; one int8
+// frame of (32768, 29491): 539 us, 599 with it).
 template <typename T, class Grp, bool VEC = true>
 __device__ __forceinline__ void op_spc(const T *__restrict__ in, uint32_t *beta, uint32_t n,
                                        uint32_t o, unsigned long long *rkey, uint32_t *rpar) {
@@ -993,7 +995,7 @@ __device__ __forceinline__ void exec_op(uint32_t kind, uint32_t n, uint32_t o, c
     case OP_R0: op_r0<Grp>(fr.beta, n, o); break;
     case OP_R1: op_r1<T, Grp>(fr.stage_in(n), fr.beta, n, o); break;
     case OP_REP: op_rep<T, Grp>(fr.stage_in(n), fr.stage(n >> 1), fr.beta, n, o); break;
-    default: op_spc<T, Grp>(fr.stage_in(n), fr.beta, n, o, fr.rkey, fr.rpar); break;
+    default: op_spc<T, Grp, false>(fr.stage_in(n), fr.beta, n, o, fr.rkey, fr.rpar); break;
     }
 }
 
