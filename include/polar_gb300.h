@@ -196,7 +196,10 @@ polar_status polar_decode_trace(const polar_code_t *code, const void *llr, int i
  *                    power of two >= 64. Wider stages live in per-CTA device
  *                    scratch.
  *   warp_stage_max   operations on nodes of size <= this run on one warp
- *                    without CTA barriers; power of two >= 2.
+ *                    without CTA barriers; power of two >= 2. Raised to the
+ *                    register subtrees of what runs: 64 leaves in the
+ *                    interpreter, the size it was compiled with in a
+ *                    specialised decoder (32 or more).
  *   ctas_per_sm      resident CTAs per SM for the persistent grid.
  *   stage_channel    1: copy each frame's LLRs into shared memory with a bulk
  *                    async copy (double buffered), 2: read them from device

@@ -156,7 +156,8 @@ polar_status choose_shape(const polar_code *c, bool is_i8, size_t n_frames, int 
         if (stage) stage = 0;
         if (kernel_smem_bytes(N, S, T, is_i8, stage) > dp.smem_optin) return POLAR_EINVAL;
     }
-    const uint32_t W = std::max<uint32_t>(u.warp_stage_max ? u.warp_stage_max : 512, kRegSubtree);
+    // at least a warp's lanes; a decoder raises it to its register subtrees
+    const uint32_t W = std::max<uint32_t>(u.warp_stage_max ? u.warp_stage_max : 512, 32);
     const size_t smem = kernel_smem_bytes(N, S, T, is_i8, stage);
     sh->threads = T;
     sh->smem_stage_max = S;
@@ -168,6 +169,11 @@ polar_status choose_shape(const polar_code *c, bool is_i8, size_t n_frames, int 
     sh->ctas_per_sm = 0;
     sh->grid = 0;
     return POLAR_OK;
+}
+
+// The shape as the interpreter runs it: register subtrees run inside warp-0 runs.
+void interpreter_shape(LaunchShape *sh) {
+    sh->warp_stage_max = std::max<uint32_t>(sh->warp_stage_max, kRegSubtree);
 }
 
 // The decoder specialised to this code and shape, if one was compiled.
@@ -303,6 +309,7 @@ polar_status decode_impl(const polar_code_t *code, const void *llr, bool is_i8,
     if (occ <= 0) {  // no specialised decoder, or it cannot be resident: interpreter
         ck = nullptr;
         sh = sh1;
+        interpreter_shape(&sh);
         occ = occupancy(device, is_i8, sh.stage_channel != 0, sh.threads, sh.smem_bytes);
     }
     st = finish_grid(c, is_i8, n_frames, device, occ, &sh);
@@ -564,6 +571,7 @@ polar_status polar_decode_noalloc(const polar_code_t *code, const float *llr, ui
     LaunchShape sh{};
     polar_status st = choose_shape(c, false, n_frames, device, &sh);
     if (st != POLAR_OK) return st;
+    interpreter_shape(&sh);
     st = finish_grid(c, false, n_frames, device,
                      occupancy(device, false, sh.stage_channel != 0, sh.threads, sh.smem_bytes), &sh);
     if (st != POLAR_OK) return st;
@@ -665,6 +673,7 @@ polar_status polar_code_get_launch(const polar_code_t *code, int is_i8, size_t n
     if (occ <= 0) {
         ck = nullptr;
         sh = sh1;
+        interpreter_shape(&sh);
         occ = occupancy(device, is_i8 != 0, sh.stage_channel != 0, sh.threads, sh.smem_bytes);
     }
     st = finish_grid(c, is_i8 != 0, n, device, occ, &sh);

@@ -61,3 +61,19 @@ def test_empty_shape_leaves_the_choice_to_the_library():
     code = polar.polar_code_create(256, 100, mask)
     autotune.configure(code, "i8", {}, n)
     assert polar.polar_code_get_launch(code, True, n)["frames_per_cta"] == 4
+
+
+@pytest.mark.parametrize("i8", [False, True])
+def test_narrow_warp_stage_is_kept(i8):
+    """warp_stage_max = 32 with 32-leaf register subtrees: nodes of 64 run on the whole CTA. The
+    interpreter, whose subtrees have 64 leaves, takes 64."""
+    n = 200
+    mask, y, t = make(512, 200, n, i8)
+    code = polar.polar_code_create(512, 200, mask)
+    polar.polar_code_set_launch(code, i8, threads=64, warp_stage_max=32)
+    assert polar.polar_code_get_launch(code, i8, n)["warp_stage_max"] == 64
+    check_bits(code, mask, y, t, i8, n)
+    polar.polar_code_compile(code, i8, n, 32)
+    launch = polar.polar_code_get_launch(code, i8, n)
+    assert launch["unrolled"] == 32 and launch["warp_stage_max"] == 32
+    check_bits(code, mask, y, t, i8, n)
