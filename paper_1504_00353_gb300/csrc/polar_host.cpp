@@ -73,6 +73,8 @@ polar_status ensure_device(polar_code *c, int device, DeviceState **out) {
     return POLAR_OK;
 }
 
+constexpr size_t kSmemPerSm = 228 * 1024;  // of which every resident CTA takes 1 KB more than it asks for
+
 struct DeviceProps {
     int sms = 0;
     int max_blocks_per_sm = 32;
@@ -193,6 +195,14 @@ CompiledKernel *find_compiled(polar_code *c, bool is_i8, const LaunchShape &sh) 
 // (8192, 6000) 104 vs 74 us for 2,560; (32768, 20000) 447 vs 263 us for 2,000).
 constexpr size_t kMultiFramesPerSm = 12;
 
+// Frames per SM that the library's own several-frames shape has to hold by its shared
+// memory: below, too few warps are in flight to cover one another's waits, and the
+// CTA-wide one-frame form is faster. N = 2^17 holds 12 (int8) and 8 (float32): 4,000
+// frames of (131072, 111411) take 2,436 and 5,494 us with one frame per CTA, 2,158
+// and 5,253 with four. N = 2^18 holds four: 5,246 and 11,764 us with one, 8,390 and
+// 15,673 with four (before the four-frames form: 6,949 and 14,122).
+constexpr size_t kMinMultiResident = 8;
+
 // The several-frames-per-CTA form of a throughput shape: F warps, each with its
 // own frame, shared-memory region and scratch; channel read in place. It is the
 // shape of a handle that asks for it (polar_code_set_frames_per_cta, one warp per
@@ -217,6 +227,7 @@ bool multi_frame_shape(const polar_code *c, bool is_i8, size_t n_frames, int dev
     const uint32_t es = is_i8 ? 1 : 4;
     const size_t per_frame = (kernel_smem_bytes(c->N, S, 32, is_i8, false) + 127) / 128 * 128;
     if (per_frame * F > device_props(device).smem_optin) return false;
+    if (u.frames_per_cta == 0 && kSmemPerSm / (per_frame * F + 1024) * F < kMinMultiResident) return false;
     const size_t g = (c->N / 2 > S) ? size_t(c->N) - 2 * size_t(S) : 0;
     sh->smem_stage_max = S;
     sh->scratch_elems_per_cta = g ? ((g * es + 127) / 128 * 128) / es : 0;
@@ -768,7 +779,7 @@ polar_status polar_code_compile_ex(polar_code_t *code, int is_i8, size_t n_frame
     const size_t per_cta = sh.smem_bytes + 1024;
     const size_t groups = (n_frames + F - 1) / F;
     gsh.ctas_per_sm = static_cast<uint32_t>(std::max<size_t>(
-        1, std::min<size_t>({size_t(228 * 1024) / per_cta, size_t(2048 / sh.threads),
+        1, std::min<size_t>({kSmemPerSm / per_cta, size_t(2048 / sh.threads),
                              size_t(dp.max_blocks_per_sm),
                              size_t(groups + dp.sms - 1) / std::max(dp.sms, 1)})));
     if (code->user[is_i8 ? 1 : 0].ctas_per_sm)

@@ -77,3 +77,22 @@ def test_narrow_warp_stage_is_kept(i8):
     launch = polar.polar_code_get_launch(code, i8, n)
     assert launch["unrolled"] == 32 and launch["warp_stage_max"] == 32
     check_bits(code, mask, y, t, i8, n)
+
+
+@pytest.mark.parametrize("i8", [False, True])
+@pytest.mark.parametrize("N,frames", [(1 << 16, 4), (1 << 18, 1)])
+def test_long_codes_keep_frames_in_flight(N, frames, i8):
+    """The library's own shape takes several frames per CTA only where shared memory then still
+    holds eight frames per SM: not for N = 2^18, whose bits alone are 32 KB a frame."""
+    mask = np.ones(N, np.uint8)
+    mask[N // 2:] = 0  # a short operation list
+    mask[N // 2::4096] = 1
+    K, n = int((mask == 0).sum()), 12 * sms()
+    code = polar.polar_code_create(N, K, mask)
+    polar.polar_code_compile(code, i8, n)
+    launch = polar.polar_code_get_launch(code, i8, n)
+    assert launch["unrolled"] and launch["frames_per_cta"] == frames
+    rng = np.random.default_rng(5)
+    y = rng.integers(-127, 128, (80, N)).astype(np.int8 if i8 else np.float32)
+    t = torch.from_numpy(y).cuda()
+    check_bits(code, mask, y, t, i8, 80)
