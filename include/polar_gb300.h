@@ -248,6 +248,9 @@ polar_status polar_code_get_launch(const polar_code_t *code, int is_i8, size_t n
  * instead of the operation-list interpreter; results are bit-identical.
  *   reg_subtree  subtrees of at most this many leaves (power of two, 32..1024;
  *                0 = 256) are decoded entirely in the registers of one warp.
+ * Of a handle whose whole launch shape is left to the library, a full batch of
+ * N >= 2^14 builds two decoders side by side: one for full batches and one for
+ * the smaller batches that the handle may also be given.
  * n_frames = 0 releases every specialised decoder of that LLR type. A decoder
  * already compiled for the same launch shape is kept (release first to build
  * one with another reg_subtree).

@@ -9,11 +9,15 @@
 #include <climits>
 #include <cstdint>
 #include <cstring>
+#include <exception>
 #include <map>
 #include <memory>
 #include <mutex>
 #include <new>
+#include <string>
+#include <thread>
 #include <tuple>
+#include <utility>
 #include <vector>
 
 #include "polar_gb300.h"
@@ -178,22 +182,28 @@ void interpreter_shape(LaunchShape *sh) {
     sh->warp_stage_max = std::max<uint32_t>(sh->warp_stage_max, kRegSubtree);
 }
 
+CompiledKey key_of(bool is_i8, const LaunchShape &sh) {
+    return CompiledKey{is_i8, sh.threads, sh.smem_stage_max, sh.warp_stage_max, sh.stage_channel,
+                       std::max<uint32_t>(sh.frames_per_cta, 1)};
+}
+
 // The decoder specialised to this code and shape, if one was compiled.
 CompiledKernel *find_compiled(polar_code *c, bool is_i8, const LaunchShape &sh) {
     std::lock_guard<std::mutex> g(c->mu);
-    auto it = c->compiled.find(CompiledKey{is_i8, sh.threads, sh.smem_stage_max,
-                                           sh.warp_stage_max, sh.stage_channel,
-                                           std::max<uint32_t>(sh.frames_per_cta, 1)});
+    auto it = c->compiled.find(key_of(is_i8, sh));
     return it == c->compiled.end() ? nullptr : &it->second;
 }
 
 // Frames per SM from which the library's own choice for a specialised decoder is
-// several frames per CTA, one per warp. Below, the SMs are not full and a frame
-// is faster with a CTA of its own: 1,280 frames (8 per SM) take the same time or up
-// to 20 % less with one frame per CTA (int8 (2048, 1707) 21.3 vs 21.2 us, (32768,
-// 27000) 134 vs 149), 2,000 and more up to 45 % less with four (25.0 vs 22.8 us;
-// (8192, 6000) 104 vs 74 us for 2,560; (32768, 20000) 447 vs 263 us for 2,000).
+// several frames per CTA, one per warp. Below, the SMs are not full and a frame is as
+// fast or faster with a CTA of its own: 1,216 frames (8 per SM) of int8 (8192, 4096)
+// 45 vs 49 us, (32768, 27000) 111 vs 123, float32 (4096, 3500) 18.5 vs 24.7; 2,500
+// frames take up to 40 % less with four (int8 (8192, 7000) 62 vs 44 us, (32768, 27000)
+// 230 vs 181, float32 (32768, 16384) 757 vs 634).
 constexpr size_t kMultiFramesPerSm = 12;
+// Frames per SM that the one-frame decoder built beside a several-frames one is meant
+// for (its register budget): more than these would not all be resident.
+constexpr size_t kOneFramePerSm = 8;
 
 // Frames per SM that the library's own several-frames shape has to hold by its shared
 // memory: below, too few warps are in flight to cover one another's waits, and the
@@ -238,28 +248,25 @@ bool multi_frame_shape(const polar_code *c, bool is_i8, size_t n_frames, int dev
     return true;
 }
 
-// Whether the library's own choice prefers one frame per CTA for n_frames frames
-// (a handle that asks for several frames per CTA always prefers them).
+// Whether the library's own choice builds one frame per CTA for n_frames frames
+// (a handle that asks for several frames per CTA always gets them).
 bool prefer_one_frame(const polar_code *c, bool is_i8, size_t n_frames, int device) {
     return c->user[is_i8 ? 1 : 0].frames_per_cta == 0 &&
            n_frames < kMultiFramesPerSm * static_cast<size_t>(device_props(device).sms);
 }
 
-// The specialised decoder for this decode: of the shapes with one and with several
-// frames per CTA the preferred one if it was compiled, else the other; *sh becomes
-// the shape of what runs.
-CompiledKernel *pick_compiled(polar_code *c, bool is_i8, size_t n_frames, int device,
-                              LaunchShape *sh) {
-    CompiledKernel *one = find_compiled(c, is_i8, *sh);
-    if (one && prefer_one_frame(c, is_i8, n_frames, device)) return one;
-    LaunchShape msh = *sh;
-    if (multi_frame_shape(c, is_i8, n_frames, device, &msh)) {
-        if (CompiledKernel *ck = find_compiled(c, is_i8, msh)) {
-            *sh = msh;
-            return ck;
-        }
-    }
-    return one;
+// Whether the library's own choice builds the one-frame decoder beside the
+// several-frames one, for the smaller batches that a handle compiled for a full
+// one is also given (a partial last batch, the chunks of polar_decode_host).
+// From N = 2^14 on: there a frame gains more from a CTA of its own than four frames
+// save by sharing their code ((32768, 27000), 160 frames: int8 95 vs 125 us, float32
+// 82 vs 157; 1,000: 103 vs 132 and 197 vs 242; with the four-frames decoder alone such
+// float32 batches were slower than before that form existed, 135 us). It costs compile
+// time, 5.5 -> 8.9 s for that int8 code. Shorter int8 codes are within 10 % either way,
+// and shorter float32 codes never were slower than before ((8192, 6000), 160 frames: 50
+// us then, 41 now).
+bool wants_both_shapes(const polar_code *c, bool is_i8) {
+    return c->user[is_i8 ? 1 : 0].frames_per_cta == 0 && c->N >= (1u << 14);
 }
 
 int compiled_occupancy(polar_code *c, CompiledKernel *ck, int device, const LaunchShape &sh) {
@@ -273,6 +280,25 @@ int compiled_occupancy(polar_code *c, CompiledKernel *ck, int device, const Laun
     std::lock_guard<std::mutex> g(c->mu);
     ck->occupancy[device] = n;
     return n;
+}
+
+// The specialised decoder for this decode: of the shapes with one and with several
+// frames per CTA the preferred one if it was compiled, else the other; *sh becomes
+// the shape of what runs. One frame per CTA is preferred as long as all frames are
+// resident at once: a second wave takes as long as the first.
+CompiledKernel *pick_compiled(polar_code *c, bool is_i8, size_t n_frames, int device,
+                              LaunchShape *sh) {
+    CompiledKernel *one = find_compiled(c, is_i8, *sh);
+    LaunchShape msh = *sh;
+    CompiledKernel *several =
+        multi_frame_shape(c, is_i8, n_frames, device, &msh) ? find_compiled(c, is_i8, msh) : nullptr;
+    if (!several) return one;
+    if (one && prefer_one_frame(c, is_i8, n_frames, device) &&
+        n_frames <= static_cast<size_t>(compiled_occupancy(c, one, device, *sh)) *
+                        static_cast<size_t>(device_props(device).sms))
+        return one;
+    *sh = msh;
+    return several;
 }
 
 // Fill ctas_per_sm and grid from the resident-CTA count of the kernel used.
@@ -294,6 +320,79 @@ polar_status cuda_status(cudaError_t e) {
     if (e == cudaSuccess) return POLAR_OK;
     if (e == cudaErrorMemoryAllocation) return POLAR_ENOMEM;
     return POLAR_ECUDA;
+}
+
+// A decoder to build: its launch shape and the largest batch it is meant for.
+struct CompileJob {
+    LaunchShape sh;
+    size_t n_frames;
+    CompiledKernel ck;
+    std::string log;
+    cudaError_t e = cudaSuccess;
+};
+
+void compile_one(const polar_code *code, bool is_i8, int device, uint32_t reg_subtree,
+                 uint32_t outline, CompileJob *j) {
+    try {
+        // register subtrees always run inside warp-0 runs
+        LaunchShape gsh = j->sh;
+        gsh.warp_stage_max = std::max(gsh.warp_stage_max, reg_subtree);
+        // resident CTAs the shared-memory footprint allows: the register budget of
+        // the generated kernel is capped so that many fit
+        const DeviceProps dp = device_props(device);
+        const size_t F = std::max<uint32_t>(gsh.frames_per_cta, 1);
+        const size_t per_cta = gsh.smem_bytes + 1024, groups = (j->n_frames + F - 1) / F;
+        gsh.ctas_per_sm = static_cast<uint32_t>(std::max<size_t>(
+            1, std::min<size_t>({size_t(228 * 1024) / per_cta, size_t(2048 / gsh.threads),
+                                 size_t(dp.max_blocks_per_sm),
+                                 size_t(groups + dp.sms - 1) / std::max(dp.sms, 1)})));
+        const uint32_t cap = code->user[is_i8 ? 1 : 0].ctas_per_sm;
+        if (cap) gsh.ctas_per_sm = std::min(gsh.ctas_per_sm, cap);
+        j->ck.reg_subtree = reg_subtree;
+        j->ck.outline = outline;
+        j->e = cudaSetDevice(device);  // of this thread
+        if (j->e == cudaSuccess)
+            j->e = compile_source(generate_source(*code, is_i8, gsh, reg_subtree, outline), &j->ck, &j->log);
+    } catch (const std::bad_alloc &) {
+        j->e = cudaErrorMemoryAllocation;
+    }
+}
+
+// Build the decoders that the handle does not have yet, side by side, and keep
+// them if all of them compile.
+polar_status compile_shapes(polar_code *code, bool is_i8, int device, uint32_t reg_subtree,
+                            uint32_t outline, std::vector<CompileJob> jobs) {
+    jobs.erase(std::remove_if(jobs.begin(), jobs.end(),
+                              [&](const CompileJob &j) { return find_compiled(code, is_i8, j.sh); }),
+               jobs.end());
+    if (jobs.empty()) return POLAR_OK;
+    std::vector<std::thread> others;
+    size_t started = 1;  // jobs[0] is this thread's
+    try {
+        others.reserve(jobs.size());
+        for (; started < jobs.size(); ++started)
+            others.emplace_back(compile_one, code, is_i8, device, reg_subtree, outline, &jobs[started]);
+    } catch (const std::exception &) {  // no thread to be had: the rest one after another
+    }
+    compile_one(code, is_i8, device, reg_subtree, outline, &jobs[0]);
+    for (size_t i = started; i < jobs.size(); ++i)
+        compile_one(code, is_i8, device, reg_subtree, outline, &jobs[i]);
+    for (std::thread &t : others) t.join();
+    cudaError_t e = cudaSuccess;
+    std::string log;
+    for (const CompileJob &j : jobs) {
+        log += j.log;
+        if (e == cudaSuccess) e = j.e;
+    }
+    std::lock_guard<std::mutex> g(code->mu);
+    code->compile_log = log;
+    for (CompileJob &j : jobs) {
+        if (e == cudaSuccess) code->compiled[key_of(is_i8, j.sh)] = j.ck;
+        else if (j.ck.lib) cudaLibraryUnload(j.ck.lib);
+    }
+    if (e == cudaSuccess) return POLAR_OK;
+    cudaGetLastError();
+    return cuda_status(e);
 }
 
 polar_status decode_impl(const polar_code_t *code, const void *llr, bool is_i8,
@@ -761,43 +860,20 @@ polar_status polar_code_compile_ex(polar_code_t *code, int is_i8, size_t n_frame
         }
         return POLAR_OK;
     }
-    LaunchShape sh{};
-    polar_status st = choose_shape(code, is_i8 != 0, n_frames, device, &sh);
+    LaunchShape one{};
+    polar_status st = choose_shape(code, is_i8 != 0, n_frames, device, &one);
     if (st != POLAR_OK) return st;
-    if (!prefer_one_frame(code, is_i8 != 0, n_frames, device))
-        multi_frame_shape(code, is_i8 != 0, n_frames, device, &sh);
-    const uint32_t F = std::max<uint32_t>(sh.frames_per_cta, 1);
-    const CompiledKey key{is_i8 != 0, sh.threads, sh.smem_stage_max, sh.warp_stage_max,
-                          sh.stage_channel, F};
-    if (find_compiled(code, is_i8 != 0, sh)) return POLAR_OK;
-    // register subtrees always run inside warp-0 runs
-    LaunchShape gsh = sh;
-    gsh.warp_stage_max = std::max(sh.warp_stage_max, reg_subtree);
-    // resident CTAs the shared-memory footprint allows: the register budget of
-    // the generated kernel is capped so that many fit
-    const DeviceProps dp = device_props(device);
-    const size_t per_cta = sh.smem_bytes + 1024;
-    const size_t groups = (n_frames + F - 1) / F;
-    gsh.ctas_per_sm = static_cast<uint32_t>(std::max<size_t>(
-        1, std::min<size_t>({kSmemPerSm / per_cta, size_t(2048 / sh.threads),
-                             size_t(dp.max_blocks_per_sm),
-                             size_t(groups + dp.sms - 1) / std::max(dp.sms, 1)})));
-    if (code->user[is_i8 ? 1 : 0].ctas_per_sm)
-        gsh.ctas_per_sm = std::min(gsh.ctas_per_sm, code->user[is_i8 ? 1 : 0].ctas_per_sm);
-    CompiledKernel ck;
-    ck.reg_subtree = reg_subtree;
-    ck.outline = outline;
-    std::string log;
-    const std::string src = generate_source(*code, is_i8 != 0, gsh, reg_subtree, outline);
-    const cudaError_t e = compile_source(src, &ck, &log);
-    std::lock_guard<std::mutex> g(code->mu);
-    code->compile_log = log;
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        return cuda_status(e);
+    std::vector<CompileJob> jobs;
+    LaunchShape several = one;
+    if (!prefer_one_frame(code, is_i8 != 0, n_frames, device) &&
+        multi_frame_shape(code, is_i8 != 0, n_frames, device, &several)) {
+        jobs.push_back({several, n_frames});
+        if (wants_both_shapes(code, is_i8 != 0))
+            jobs.push_back({one, kOneFramePerSm * static_cast<size_t>(device_props(device).sms)});
+    } else {
+        jobs.push_back({one, n_frames});
     }
-    code->compiled[key] = ck;
-    return POLAR_OK;
+    return compile_shapes(code, is_i8 != 0, device, reg_subtree, outline, std::move(jobs));
 }
 
 const char *polar_code_compile_log(const polar_code_t *code) {

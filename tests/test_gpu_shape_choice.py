@@ -79,14 +79,20 @@ def test_narrow_warp_stage_is_kept(i8):
     check_bits(code, mask, y, t, i8, n)
 
 
+def short_list(N):
+    """A mask with a short operation list."""
+    mask = np.ones(N, np.uint8)
+    mask[N // 2:] = 0
+    mask[N // 2::4096] = 1
+    return mask
+
+
 @pytest.mark.parametrize("i8", [False, True])
 @pytest.mark.parametrize("N,frames", [(1 << 16, 4), (1 << 18, 1)])
 def test_long_codes_keep_frames_in_flight(N, frames, i8):
     """The library's own shape takes several frames per CTA only where shared memory then still
     holds eight frames per SM: not for N = 2^18, whose bits alone are 32 KB a frame."""
-    mask = np.ones(N, np.uint8)
-    mask[N // 2:] = 0  # a short operation list
-    mask[N // 2::4096] = 1
+    mask = short_list(N)
     K, n = int((mask == 0).sum()), 12 * sms()
     code = polar.polar_code_create(N, K, mask)
     polar.polar_code_compile(code, i8, n)
@@ -96,3 +102,30 @@ def test_long_codes_keep_frames_in_flight(N, frames, i8):
     y = rng.integers(-127, 128, (80, N)).astype(np.int8 if i8 else np.float32)
     t = torch.from_numpy(y).cuda()
     check_bits(code, mask, y, t, i8, 80)
+
+
+@pytest.mark.parametrize("i8", [False, True])
+def test_full_batch_handle_decodes_smaller_batches_one_per_cta(i8):
+    """A handle compiled for a full batch of a long code runs batches that one CTA per frame
+    holds at once with one frame per CTA, larger ones with four; the decoder of an earlier
+    compile is kept beside them."""
+    N, full = 1 << 14, 12 * sms() + 3
+    mask = short_list(N)
+    K = int((mask == 0).sum())
+    rng = np.random.default_rng(6)
+    y = rng.integers(-9, 10, (full, N)).astype(np.int8 if i8 else np.float32)
+    t = torch.from_numpy(y).cuda()
+    code = polar.polar_code_create(N, K, mask)
+    for first in (full, 1):  # alone, then beside the batch-1 decoder
+        if first == 1:
+            polar.polar_code_compile(code, i8, 0)
+            polar.polar_code_compile(code, i8, 1)
+        polar.polar_code_compile(code, i8, full)
+        for n, frames in ((full, 4), (12 * sms() - 1, 4), (8 * sms(), 1), (sms() + 1, 1), (1, 1)):
+            launch = polar.polar_code_get_launch(code, i8, n)
+            assert launch["frames_per_cta"] == frames, n
+            assert bool(launch["unrolled"]) == (n > 1 or first == 1)
+            check_bits(code, mask, y, t, i8, n)
+    host = polar.polar_decode_host(code, t[:sms() * 8].cpu()).numpy()  # eight chunks
+    assert np.array_equal(host[:2], oracle.decode_batch(mask, y, frames=np.arange(2)))
+    assert np.array_equal(host, (polar.polar_decode_i8 if i8 else polar.polar_decode)(code, t[:sms() * 8]).cpu().numpy())
