@@ -111,7 +111,7 @@ struct polar_code {
     std::vector<uint8_t> frozen;
     std::vector<uint32_t> frozen_prefix;  // frozen count in [0, i)
     std::vector<uint32_t> info_idx;       // A in increasing order
-    std::vector<polar::HostOp> ops;       // interpreter list (register subtrees <= 32)
+    std::vector<polar::HostOp> ops;       // interpreter list (register subtrees <= kRegSubtree)
     std::vector<uint32_t> trace_off;      // per op (F/G/G_0R), floats
     size_t trace_len = 0;
     uint32_t NW = 1, KW = 0;

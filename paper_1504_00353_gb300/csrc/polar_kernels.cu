@@ -58,7 +58,7 @@ __device__ __forceinline__ void trace_store(uint32_t kind, uint32_t n, uint32_t 
 // their lives between subtrees. Left as they were, they stayed allocated across the
 // memory-level operations and those spilled: 408 (float32) and 660 (int8) bytes, now
 // none. 1,000 frames of (1024, 512), float32 92 us before this layout, 82 with the
-// spills, 72 now; int8 96, 82, 70; 4,000 of (32768, 29491) int8 2,935, 2,997, 2,515.
+// spills, 72 now; int8 96, 82, 70; 4,000 of (32768, 29491) int8 2,935, 2,997, 2,574.
 template <typename T, bool TRACE>
 struct RegTree {
     using Sub = RegSub<T, kRegSubtree, true>;

@@ -213,8 +213,6 @@ __device__ __forceinline__ float op_g(float a, float b, uint32_t bit) { return g
 __device__ __forceinline__ int op_g(int a, int b, uint32_t bit) { return g_i8s(a, b, bit); }
 __device__ __forceinline__ float op_add(float a, float b) { return a + b; }
 __device__ __forceinline__ int op_add(int a, int b) { return sat127(a + b); }
-__device__ __forceinline__ uint32_t mag_bits(float a) { return __float_as_uint(fabsf(a)); }
-__device__ __forceinline__ uint32_t mag_bits(int a) { return static_cast<uint32_t>(abs(a)); }
 
 // Four int8 lanes per 32-bit word, computed as two f16x2 pairs. Every int8
 // value and every sum of two of them is an integer of magnitude <= 254, exact
@@ -405,8 +403,6 @@ __device__ __forceinline__ void discard_l2(const void *p, uint32_t bytes) {
 }
 
 // ---------------------------------------------------------------- beta helpers
-
-__device__ __forceinline__ uint32_t low_mask(uint32_t n) { return n >= 32 ? kFull : ((1u << n) - 1u); }
 
 // Replace bits [off, off+n) (n <= 32, inside one word) with the low n bits of v.
 __device__ __forceinline__ void write_field(uint32_t *beta, uint32_t off, uint32_t n, uint32_t v) {
