@@ -102,6 +102,7 @@ def frames_for(N: int, sms: int) -> int:
     return int(max(sms * 48, min(1 << 17, (1 << 26) // N)))
 
 
+# local_leaves: of older table entries, changes nothing any more
 SHAPE_KEYS = ("threads", "smem_stage_max", "warp_stage_max", "ctas_per_sm", "stage_channel",
               "reg_subtree", "frames_per_cta", "local_leaves", "compile_form")
 SHAPE_DEFAULTS = dict(ctas_per_sm=0, stage_channel=2, reg_subtree=256, frames_per_cta=1,
@@ -125,8 +126,7 @@ def apply_shape(code, dtype: str, shape: dict, n_frames: int):
                                 ctas_per_sm=sh["ctas_per_sm"], stage_channel=sh["stage_channel"])
     polar.polar_code_set_frames_per_cta(code, dtype == "i8", sh["frames_per_cta"])
     polar.polar_code_compile(code, dtype == "i8", n_frames, sh["reg_subtree"],
-                             COMPILE_FORM[sh["compile_form"]] |
-                             (polar.COMPILE_LOCAL_LEAVES if sh["local_leaves"] else 0))
+                             COMPILE_FORM[sh["compile_form"]])
 
 
 def _compile(N, K, mask, dtype, shape, n_frames):
@@ -254,8 +254,6 @@ class CodeTuner:
         self.measure([dict(cur, reg_subtree=r) for r in (256, 512, 1024)])
         cur, _ = self.best()
         self.measure([dict(cur, stage_channel=c) for c in (1, 2)])
-        cur, _ = self.best()
-        self.measure([dict(cur, local_leaves=v) for v in (0, 1)])
         return self.best()
 
     def tune(self, threads_options=THREADS, fixed_threads=None, tune_ctas=True) -> tuple[dict, float]:
@@ -514,7 +512,7 @@ def configure(code, dtype: str, shape: dict, n_frames: int, interpreter: bool = 
     # an empty shape leaves the frames per CTA of a handle as they are: the library's choice
     # unless the program has set them
     fpc = sh.pop("frames_per_cta", 1 if sh else None)
-    local = polar.COMPILE_LOCAL_LEAVES if sh.pop("local_leaves", 0) else 0
+    sh.pop("local_leaves", None)
     tuned_form = sh.pop("compile_form", "auto")
     if form == "auto":  # an explicit form from the caller wins over the table's
         form = tuned_form
@@ -522,7 +520,7 @@ def configure(code, dtype: str, shape: dict, n_frames: int, interpreter: bool = 
     if fpc is not None:
         polar.polar_code_set_frames_per_cta(code, dtype == "i8", fpc)
     if not interpreter:
-        polar.polar_code_compile(code, dtype == "i8", n_frames, reg, COMPILE_FORM[form] | local)
+        polar.polar_code_compile(code, dtype == "i8", n_frames, reg, COMPILE_FORM[form])
 
 
 def batch_shape(dtype: str):
