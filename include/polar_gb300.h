@@ -303,7 +303,8 @@ typedef struct polar_batch polar_batch_t;
  *   warp_stage_max  per code, the largest node handled by warp 0 alone: the
  *                   tree depth at which work switches from CTA-wide to
  *                   warp-level (power of two; NULL or 0 entries = 2048;
- *                   raised to 256, the register-resident subtree size).
+ *                   raised to the register-resident subtree size, 256 leaves
+ *                   for float32 and 512 for int8).
  *   ctas_per_sm     cap on resident CTAs (frames) per SM, which also sets the
  *                   register budget of the kernel (0 = as many as shared
  *                   memory allows, at most 32).
